@@ -164,6 +164,43 @@ static int prime_state(pdn_ctx *ctx) {
   return PDN_OK;
 }
 
+// Bound on the strain components below which no point with the initial
+// history yields or reaches a damage onset (Mat::e_tol).  With every normal
+// component and engineering shear at most t, the tensor's Frobenius norm n is
+// at most sqrt(4.5) t, the same in ply axes, and each criterion of Algorithm 4
+// is bounded by a function of n: |e_ii| <= n; the 12, 13 shears together at
+// most sqrt(2) n; |sigma_ii| at most the norm of the stiffness row times n.
+// With the smallest seeded strengths and 0.1 % to spare for the rounding of
+// the criteria; unbounded when both laws are off.
+double elastic_strain_bound(const pdn_material &m, const double (&C)[3][3], double kT, int damage_on,
+                            int plasticity_on) {
+  double n = 1e30;
+  if (plasticity_on) n = std::min(n, m.Sp / (m.G12 * std::sqrt(2.0)));
+  if (damage_on) {
+    const double lo = 1.0 - std::fabs(m.spread);
+    const double r1 = std::sqrt(C[0][0] * C[0][0] + C[0][1] * C[0][1] + C[0][2] * C[0][2]);
+    const double r2 = std::sqrt(C[0][1] * C[0][1] + C[1][1] * C[1][1] + C[1][2] * C[1][2]);
+    n = std::min(n, std::min(m.XT * lo / m.E1, m.XC / r1));
+    const double a0 = m.alpha0_deg * M_PI / 180.0;
+    const double ST = m.YC * std::cos(a0) * (std::sin(a0) + std::cos(a0) / std::tan(2.0 * a0));
+    const double g = m.GYT / m.GSL, sl = std::sqrt(2.0) * std::max(m.G12, m.G13) / (m.SL * lo);
+    const double sq = std::sqrt(2.0) * m.G23 / ST, st = r2 * kT / ST, yt = r2 / (m.YT * lo);
+    auto matrix = [&](double x) {  // largest of the two matrix criteria at norm x
+      const double sh = (sl * sl + sq * sq) * x * x;
+      return std::max(std::fabs(1.0 - g) * yt * x + std::fabs(g) * yt * yt * x * x + sh, st * st * x * x + sh);
+    };
+    double hi = n, b = 0.0;
+    for (int k = 0; k < 200; ++k) {
+      const double mid = 0.5 * (b + hi);
+      if (matrix(mid) <= 1.0) b = mid;
+      else hi = mid;
+    }
+    n = b;
+  }
+  const double t = 0.999 * n / std::sqrt(4.5);
+  return t > 0.0 && std::isfinite(t) ? t : 0.0;
+}
+
 // Material constants in precision T from the double-precision record.
 template <typename T>
 int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_plies, int damage_on,
@@ -243,6 +280,7 @@ int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_pl
   M.eta = (T)m.eta;
   M.onset_floor = (T)(0.999 * std::min(KI * D3o * D3o, Ksh * Dsho * Dsho));
   M.spread = (T)m.spread;
+  M.e_tol = (T)elastic_strain_bound(m, C, ca * (sa + ca / t2), damage_on, plasticity_on);
   M.seed = m.seed;
   M.damage_on = damage_on;
   M.plasticity_on = plasticity_on;
@@ -253,6 +291,30 @@ int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_pl
   }
   return PDN_OK;
 }
+
+}  // namespace
+
+namespace pdn {
+void ply_stiffness(const Mat<double> &M, int p, double (&q)[13]) {
+  const double c = M.ply_c[p], s = M.ply_s[p], c2 = c * c, s2 = s * s, cs = c * s;
+  // ply strains (11 22 33 12 | 13 23, engineering) of the global ones (xx yy
+  // zz xy | xz yz); the stiffness is R^T C R with the same R
+  const double R[4][4] = {{c2, s2, 0, cs}, {s2, c2, 0, -cs}, {0, 0, 1, 0}, {-2 * cs, 2 * cs, 0, c2 - s2}};
+  const double C[4][4] = {{M.C11, M.C12, M.C13, 0}, {M.C12, M.C22, M.C23, 0}, {M.C13, M.C23, M.C33, 0}, {0, 0, 0, M.G12}};
+  double K[4][4];
+  for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < 4; ++j) {
+      K[i][j] = 0.0;
+      for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < 4; ++b) K[i][j] += R[a][i] * C[a][b] * R[b][j];
+    }
+  const double out[13] = {K[0][0], K[0][1], K[0][2], K[0][3], K[1][1], K[1][2], K[1][3], K[2][2], K[2][3], K[3][3],
+                          s2 * M.G13 + c2 * M.G23, cs * (M.G13 - M.G23), c2 * M.G13 + s2 * M.G23};
+  for (int k = 0; k < 13; ++k) q[k] = out[k];
+}
+}  // namespace pdn
+
+namespace {
 
 // Hex8 geometry on the host (set-up only): det J and N_a at the 2x2x2 points.
 // Shape functions and their natural derivatives at the 2x2x2 Gauss points,
@@ -966,6 +1028,7 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     char *iw, *rDn[2];
     uint32_t *rank;
     int8_t *ply;
+    char *box, *ply_q;
     char *X4, *imass, *u4[2], *hist[2], *rD[2], *fe;
     uint8_t *nflag, *act[2], *rel, *rmark_e, *rmark_n, *pflag[2], *cflag[2];
     double *Xs, *mass, *d[2], *v[2], *nrm, *lam, *trial, *fhist, *fout;
@@ -982,6 +1045,8 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     P.coh = A.take<int32_t>(sizeof(int32_t) * nc1 * 8);
     P.ply = A.take<int8_t>((nh + 15) & ~int64_t(15));  // whole 16-byte words (read as words)
     P.X4 = A.take<char>(ts * 4 * nn);
+    P.box = A.take<char>(all_boxes ? ts * 4 * nh : 32);
+    P.ply_q = A.take<char>(sizeof(double) * 16 * kMaxPlies);
     P.nflag = A.take<uint8_t>((nn + 3) & ~int64_t(3));  // whole 4-byte words (the sweep copies words)
     P.surf = A.take<int32_t>(sizeof(int32_t) * ns1);
     P.surf_of = A.take<int32_t>(sizeof(int32_t) * nn);
@@ -1170,6 +1235,8 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     D.coh = d_coh;
     D.ply = d_ply;
     D.X4 = reinterpret_cast<const V4 *>(d_X4);
+    D.box = reinterpret_cast<const V4 *>(P.box);
+    D.ply_q = reinterpret_cast<const T *>(P.ply_q);
     D.nflag = d_nflag;
     D.surf = d_surf;
     D.surf_of = d_surf_of;
@@ -1232,10 +1299,20 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     D.ell = ell ? 1 : 0;
     D.surf_base = surf_base;
   };
-  if (fp64)
+  if (fp64) {
     wire(ctx->Dd, double{});
-  else
+    std::vector<double> q((size_t)kPlyStride<double> * mesh->n_plies);
+    ply_table(ctx->Md, mesh->n_plies, q.data());
+    chk(up(P.ply_q, q.data(), sizeof(double) * q.size()));
+    if (all_boxes) chk(launch_box_records(ctx->Dd, reinterpret_cast<double4_32a *>(P.box), ctx->stream));
+  } else {
     wire(ctx->Df, float{});
+    std::vector<float> q((size_t)kPlyStride<float> * mesh->n_plies);
+    ply_table(ctx->Md, mesh->n_plies, q.data());
+    chk(up(P.ply_q, q.data(), sizeof(float) * q.size()));
+    if (all_boxes) chk(launch_box_records(ctx->Df, reinterpret_cast<float4 *>(P.box), ctx->stream));
+  }
+  if (e != cudaSuccess) return die(PDN_E_CUDA, std::string("ply and box tables: ") + cudaGetErrorString(e));
   ctx->rmark_e_buf = d_rmark_e;
   ctx->rmark_n_buf = d_rmark_n;
   {

@@ -34,6 +34,14 @@ using namespace detail;
 
 enum TileKind : int32_t { TK_CONTACT = 0, TK_HEX = 1, TK_COH = 2, TK_GATHER = 3, TK_TAIL = 4 };
 
+// The hexes [first, end) of a plate, out of line: the element code then has the
+// launch's whole register budget to itself (inlined into the tile loop it
+// spilled 650 bytes a thread at 128 registers).
+template <typename T, bool BOX>
+__device__ __noinline__ void batch_hex(const Dev<T> &D, const Mat<T> &M, int64_t first, int64_t end, int mode) {
+  hex_item<T, BOX>(D, M, first, end, mode);
+}
+
 // The gather of one node of a plate: with the plate's interfaces as node
 // pairs (Dev::ipair) the gather evaluates them too, and the plate has no
 // interface tiles.
@@ -168,9 +176,9 @@ __global__ void __launch_bounds__(kBatchBlock, MINB) k_batch(BatchArgs<T> A) {
           case TK_HEX:
             if (mode < MODE_DONE) {
               if (sD.all_boxes)
-                for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) hex_item<T, true>(sD, sM, i, mode);
+                batch_hex<T, true>(sD, sM, tl.z, tl.w, mode);
               else
-                for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) hex_item<T, false>(sD, sM, i, mode);
+                batch_hex<T, false>(sD, sM, tl.z, tl.w, mode);
             }
             break;
           case TK_COH:
@@ -303,9 +311,9 @@ __global__ void __launch_bounds__(kBatchBlock, MINB) k_batch_flow(FlowArgs<T> A)
       case TK_HEX:
         if (mode < MODE_DONE) {
           if (sD.all_boxes)
-            for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) hex_item<T, true>(sD, sM, i, mode);
+            batch_hex<T, true>(sD, sM, tl.z, tl.w, mode);
           else
-            for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) hex_item<T, false>(sD, sM, i, mode);
+            batch_hex<T, false>(sD, sM, tl.z, tl.w, mode);
         }
         break;
       case TK_COH:

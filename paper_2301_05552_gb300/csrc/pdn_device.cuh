@@ -42,6 +42,13 @@ __device__ __forceinline__ double rdiv(double a, double b) { return __ddiv_rn(a,
 __device__ __forceinline__ float rsqrt_rn(float a) { return __fsqrt_rn(a); }
 __device__ __forceinline__ double rsqrt_rn(double a) { return __dsqrt_rn(a); }
 
+// Packed FP32 pairs: one sm_100-family instruction computes both lanes, each
+// lane rounded exactly as the scalar operation.
+__device__ __forceinline__ float2 p2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+
 // Exact float <-> double conversions with integer instructions.  On this part
 // the hardware conversions issue at the FP64 rate (about 0.6 T/s, measured),
 // 30x slower than the integer pipe, and the node update needs six per node.

@@ -92,6 +92,10 @@ struct Mat {
   // interface
   T KI, Ksh, KI_D3o2, Ksh_Dsho2, KI_D3oD3c, Ksh_DshoDshc, eta, onset_floor;
   T spread;
+  // every strain component (tensor normals, engineering shears, in any axes
+  // about z) of magnitude below e_tol: no yield and no damage onset from the
+  // initial history, whatever the seeded strengths (the hex kernel's screen)
+  T e_tol;
   T ply_c[kMaxPlies], ply_s[kMaxPlies];
   uint64_t seed;
   int32_t damage_on, plasticity_on;
@@ -145,6 +149,10 @@ struct Dev {
   const int32_t *hex;      // [nh][8]
   const int32_t *coh;      // [nc][8]
   const int8_t *ply;       // [nh]
+  // box meshes (all_boxes): {1/hx, 1/hy, 1/hz, volume / 8} of each hex
+  const V4 *box;           // [nh]
+  // stiffness of each ply in global axes, 13 constants (pdn_hex.cuh)
+  const T *ply_q;          // [n_plies][kPlyStride]
   const V4 *X4;            // [nn] reference coordinates (x, y, z, 0) in T
   const uint8_t *nflag;    // [nn] bits 0-2 constraint, bit 3 contact surface
   const int32_t *surf;     // [ns]
@@ -270,7 +278,31 @@ struct Dev {
 };
 constexpr int kFlagPairShift = 4;  // node flag bits 4-6: incident interface elements
 
+// Layout of Dev::ply_q: 13 constants of 16 per ply, each stored kPlyRep times
+// in a row (twice for float: 16-byte loads then bring operand pairs of the
+// packed FP32 operations).
+template <typename T>
+constexpr int kPlyRep = sizeof(T) == 4 ? 2 : 1;
+template <typename T>
+constexpr int kPlyStride = 16 * kPlyRep<T>;
+
+// Stiffness of ply p in global axes (pdn_api.cu): xx yy zz xy block 11 12 13
+// 16 22 23 26 33 36 66, then yz-yz, yz-xz, xz-xz, for engineering shears.
+void ply_stiffness(const Mat<double> &M, int p, double (&q)[13]);
+template <typename T>
+inline void ply_table(const Mat<double> &M, int n_plies, T *out) {
+  for (int p = 0; p < n_plies; ++p) {
+    double q[13];
+    ply_stiffness(M, p, q);
+    for (int k = 0; k < 16; ++k)
+      for (int r = 0; r < kPlyRep<T>; ++r) out[p * kPlyStride<T> + k * kPlyRep<T> + r] = k < 13 ? (T)q[k] : T(0);
+  }
+}
+
 // Launchers (pdn_kernels.cu).
+// Box records (Dev::box) from the reference coordinates.
+template <typename T>
+cudaError_t launch_box_records(const Dev<T> &D, typename Vec4T<T>::type *box, cudaStream_t s);
 template <typename T>
 cudaError_t launch_pass(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_t gather_block,
                         cudaEvent_t *ev /* [6] or nullptr */, cudaStream_t side = nullptr,

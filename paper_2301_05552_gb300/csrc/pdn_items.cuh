@@ -26,6 +26,8 @@
 #define PDN_STATE_RESTRICT __restrict__
 #endif
 
+#include "pdn_hex.cuh"
+
 namespace pdn {
 namespace detail {
 
@@ -159,526 +161,18 @@ __device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mod
 }
 
 // ---------------------------------------------------------------------------
-// Packed FP32 pairs: one sm_100-family instruction computes both lanes, each
-// lane rounded exactly as the scalar operation.
-__device__ __forceinline__ float2 p2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-
-// Gauss point of lane l (0: xi < 0, 1: xi > 0) in xi-pair p (bit 0: eta > 0,
-// bit 1: zeta > 0), in the point numbering of the node signs (sgn_x/y/z).
-__host__ __device__ constexpr int pair_point(int p, int l) {
-  return ((p >> 1) << 2) + ((p & 1) ? (l ? 2 : 3) : (l ? 1 : 0));
-}
-
-// The FP32 hex8 of an axis-aligned box, two Gauss points per step.  The two
-// points of a pair differ only in the sign of xi, so the displacement
-// gradient, the Green strain, both rotations, P = S F^T and the mode-space
-// force sums run as packed pairs; the intralaminar law runs per point.
-// Same formulation as the scalar element below (Eq. fcont, Algorithm 4).
-// The compute of hex_item_box_pairs from the element's node displacements
-// ua (by node) and the x-y-z extents of the box (corner 6 minus corner 0);
-// the element's nodal forces f[8][3] are handed to store(f).
-template <typename Store>
-__device__ __forceinline__ void hex_box_pairs_core(const Dev<float> &D, const Mat<float> &M, int64_t e, int mode,
-                                                   const float (&ua)[8][3], float ex, float ey, float ez,
-                                                   bool pristine_in, int ply, Store &&store);
-
-// Nodal forces of hex e (box, FP32) at the displacement mirror of the pass,
-// handed to store(f, nd) with the element's node ids; false when a repeated
-// pass does not evaluate it.
-template <typename Store>
-__device__ __forceinline__ bool hex_box_forces(const Dev<float> &D, const Mat<float> &M, int64_t e, int mode,
-                                               Store &&store) {
-  using V4 = float4;
-  const Ctl *ctl = D.ctl;
-  if (mode == MODE_REPEAT && !repeat_take(D.rmark_e, e)) return false;
-  const int ub = (mode == MODE_FORCES) ? (ctl->dpar ^ 1) : ctl->dpar;
-  const V4 *PDN_STATE_RESTRICT U = D.u4[ub];
-  const int4 c0 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e);
-  const int4 c1 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e + 1);
-  const int nd[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-  if (!nodes_in_range(D, nd)) return false;
-  if (mode == MODE_REPEAT) repeat_mark_nodes(D.rmark_n, nd);
-  float ua[8][3];
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const V4 u = U[nd[a]];
-    ua[a][0] = u.x;
-    ua[a][1] = u.y;
-    ua[a][2] = u.z;
-  }
-  const V4 x0 = D.X4[nd[0]], x6 = D.X4[nd[6]];
-  const bool pristine_in = D.pflag[0] != nullptr && D.pflag[ctl->hpar][e] != 0;
-  hex_box_pairs_core(D, M, e, mode, ua, x6.x - x0.x, x6.y - x0.y, x6.z - x0.z, pristine_in, D.ply[e],
-                     [&](const float (&f)[8][3]) { store(f, nd); });
-  return true;
-}
-
-__device__ __forceinline__ void hex_item_box_pairs(const Dev<float> &D, const Mat<float> &M, int64_t e, int mode) {
-  if (e >= D.nh) return;
-  const uint32_t rk = D.rank != nullptr ? __ldg(D.rank + e) : 0u;
-  const int4 *pos2 = reinterpret_cast<const int4 *>(D.pos) + 2 * e;
-  hex_box_forces(D, M, e, mode, [&](const float (&f)[8][3], const int (&nd)[8]) {
-    int ps[8];
-    element_slots(D, D.hex, e, pos2, rk, ps);
-#pragma unroll
-    for (int a = 0; a < 8; ++a) D.fe[ps[a]] = make_float4(f[a][0], f[a][1], f[a][2], 0.0f);
-  });
-}
-
-template <typename Store>
-__device__ __forceinline__ void hex_box_pairs_core(const Dev<float> &D, const Mat<float> &M, int64_t e, int mode,
-                                                   const float (&ua)[8][3], float ex, float ey, float ez,
-                                                   bool pristine_in, int ply, Store &&store) {
-  const Ctl *ctl = D.ctl;
-  const int64_t nh = D.nh;
-  const int hb = ctl->hpar;
-  const float *PDN_STATE_RESTRICT hin = D.hist[hb] + e;
-  float *PDN_STATE_RESTRICT hout = D.hist[hb ^ 1] + e;
-  bool dirty = false;
-  float bm[8][3];
-  float jd[3], wd[3], vol;
-  {
-    to_modes(ua, bm);
-    const float J0 = 0.5f * ex, J1 = 0.5f * ey, J2 = 0.5f * ez;
-    const float det = J0 * (J1 * J2);
-    jd[0] = xrcp(J0);
-    jd[1] = xrcp(J1);
-    jd[2] = xrcp(J2);
-    wd[0] = det * jd[0];
-    wd[1] = det * jd[1];
-    wd[2] = det * jd[2];
-    vol = 8.0f * det;
-  }
-  const float cs = M.ply_c[ply], sn = M.ply_s[ply];
-  const float c2 = cs * cs, s2 = sn * sn, csn = cs * sn;
-  const ElemLaw<float> L = elem_law(M, e);
-  float lc = -1.0f;
-  // mode-space force sums
-  float C[8][3];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) C[m][0] = C[m][1] = C[m][2] = 0.0f;
-  const float gp = 0.57735026918962576451f;
-  const float2 xi = make_float2(-gp, gp);
-#pragma unroll 1
-  for (int p = 0; p < 4; ++p) {
-    const int gx = pair_point(p, 0), gy = pair_point(p, 1);
-    // the pair's history, in flight while the strains are computed; an
-    // element with the initial history takes it without a load (a branch,
-    // uniform over the warp wherever its elements are all pristine)
-    float2 h[7];
-    if (pristine_in) {
-#pragma unroll
-      for (int f = 0; f < 7; ++f) h[f] = p2(f < 4 ? 1.0f : 0.0f);
-    } else {
-#pragma unroll
-      for (int f = 0; f < 7; ++f) h[f] = make_float2(hin[(int64_t)(f * 8 + gx) * nh], hin[(int64_t)(f * 8 + gy) * nh]);
-    }
-    const float et = (p & 1) ? gp : -gp, ze = (p & 2) ? gp : -gp;
-    const float etze = et * ze;
-    // H = du/dX: the xi column is the same in both lanes; the eta and zeta
-    // columns are a + xi b
-    float2 H[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      H[i][0] = p2((bm[1][i] + et * bm[4][i] + ze * bm[6][i] + etze * bm[7][i]) * jd[0]);
-      const float a1 = (bm[2][i] + ze * bm[5][i]) * jd[1], b1 = (bm[4][i] + ze * bm[7][i]) * jd[1];
-      const float a2 = (bm[3][i] + et * bm[5][i]) * jd[2], b2 = (bm[6][i] + et * bm[7][i]) * jd[2];
-      H[i][1] = pfma(xi, p2(b1), p2(a1));
-      H[i][2] = pfma(xi, p2(b2), p2(a2));
-    }
-    // Green strain E = 1/2 (H + H^T + H^T H), then to ply axes (rotation about z)
-    float2 E[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = i; k < 3; ++k) {
-        float2 t = padd(H[i][k], H[k][i]);
-        t = pfma(H[0][i], H[0][k], t);
-        t = pfma(H[1][i], H[1][k], t);
-        t = pfma(H[2][i], H[2][k], t);
-        E[i][k] = pmul(p2(0.5f), t);
-      }
-    float2 ep[6];
-    ep[0] = pfma(p2(s2), E[1][1], pfma(p2(2.0f * csn), E[0][1], pmul(p2(c2), E[0][0])));
-    ep[1] = pfma(p2(c2), E[1][1], pfma(p2(-2.0f * csn), E[0][1], pmul(p2(s2), E[0][0])));
-    ep[2] = E[2][2];
-    ep[3] = pfma(p2(2.0f * csn), E[1][1], pfma(p2(2.0f * (c2 - s2)), E[0][1], pmul(p2(-2.0f * csn), E[0][0])));
-    ep[4] = pfma(p2(2.0f * sn), E[1][2], pmul(p2(2.0f * cs), E[0][2]));
-    ep[5] = pfma(p2(2.0f * cs), E[1][2], pmul(p2(-2.0f * sn), E[0][2]));
-    // the law.  Pristine points (initial history) that stay below yield and
-    // below every onset, in both lanes, keep their history and take the
-    // effective stress as nominal stress: the same tests as cdm_plastic and
-    // cdm_damage with r = 1 and no plastic strain, in packed arithmetic.
-    // Every other pair takes the full law, one point at a time.
-    float2 sm[6];
-    bool elastic = false;
-    if (pristine_in) {
-      const float2 s11 = pfma(p2(M.C13), ep[2], pfma(p2(M.C12), ep[1], pmul(p2(M.C11), ep[0])));
-      const float2 s22 = pfma(p2(M.C23), ep[2], pfma(p2(M.C22), ep[1], pmul(p2(M.C12), ep[0])));
-      const float2 s33 = pfma(p2(M.C33), ep[2], pfma(p2(M.C23), ep[1], pmul(p2(M.C13), ep[0])));
-      const float2 s12 = pmul(p2(M.G12), ep[3]), s13 = pmul(p2(M.G13), ep[4]), s23 = pmul(p2(M.G23), ep[5]);
-      bool ok = true;
-      if (M.plasticity_on) {
-        const float2 t12 = pmul(p2(M.G12), ep[3]), t13 = pmul(p2(M.G12), ep[4]);
-        const float2 tn2 = pfma(t13, t13, pmul(t12, t12));
-        const float ty2 = M.Sp * M.Sp;
-        ok = tn2.x <= ty2 && tn2.y <= ty2;
-      }
-      if (ok && M.damage_on) {
-        const float2 phiFT = pmul(pmul(p2(M.E1), ep[0]), p2(L.iXT));
-        const float2 tl2 = pfma(s13, s13, pmul(s12, s12));
-        const float2 a = pmul(s22, p2(L.iYT));
-        const float2 s23q = pmul(pmul(s23, s23), p2(M.iST2));
-        // matrix tension: (1-g) a + g a^2 + tauL^2/SL^2 + s23^2/ST^2
-        const float2 qmt = padd(pfma(tl2, p2(L.iSL2), pfma(pmul(p2(M.g), a), a, pmul(p2(M.g1), a))), s23q);
-        // matrix compression: the bound (tT^2 + s23^2)/ST^2 + tauL^2/SL^2
-        const float tTx = fmaxf(-s22.x * M.kT, 0.0f), tTy = fmaxf(-s22.y * M.kT, 0.0f);
-        const float2 tT = make_float2(tTx, tTy);
-        const float2 qmc = pfma(tl2, p2(L.iSL2), pmul(pfma(tT, tT, pmul(s23, s23)), p2(M.iST2)));
-        const float qx = s22.x >= 0.0f ? qmt.x : qmc.x, qy = s22.y >= 0.0f ? qmt.y : qmc.y;
-        const float fcx = fmaxf(-s11.x, 0.0f) * M.iXC, fcy = fmaxf(-s11.y, 0.0f) * M.iXC;
-        ok = phiFT.x <= 1.0f && phiFT.y <= 1.0f && fcx <= 1.0f && fcy <= 1.0f && qx <= 1.0f && qy <= 1.0f;
-      }
-      if (ok) {
-        sm[0] = s11;
-        sm[1] = s22;
-        sm[2] = s33;
-        sm[3] = s12;
-        sm[4] = s13;
-        sm[5] = s23;
-        elastic = true;
-      }
-    }
-    if (!elastic) {
-      float el[6], hl[7], sl[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) el[k] = ep[k].x;
-#pragma unroll
-      for (int f = 0; f < 7; ++f) hl[f] = h[f].x;
-      cdm(M, L, (const float(*)[3]) nullptr, vol, lc, el, hl, sl);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) sm[k].x = sl[k];
-#pragma unroll
-      for (int f = 0; f < 7; ++f) h[f].x = hl[f];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) el[k] = ep[k].y;
-#pragma unroll
-      for (int f = 0; f < 7; ++f) hl[f] = h[f].y;
-      cdm(M, L, (const float(*)[3]) nullptr, vol, lc, el, hl, sl);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) sm[k].y = sl[k];
-#pragma unroll
-      for (int f = 0; f < 7; ++f) h[f].y = hl[f];
-    }
-    if (!pristine_in) {
-#pragma unroll
-      for (int f = 0; f < 7; ++f) {
-        hout[(int64_t)(f * 8 + gx) * nh] = h[f].x;
-        hout[(int64_t)(f * 8 + gy) * nh] = h[f].y;
-      }
-    } else {
-      // a pair that passed the elastic test kept the initial history
-      const bool changed = !elastic &&
-                           (h[0].x > 1.0f || h[1].x > 1.0f || h[2].x > 1.0f || h[3].x > 1.0f || h[4].x != 0.0f ||
-                            h[5].x != 0.0f || h[6].x != 0.0f || h[0].y > 1.0f || h[1].y > 1.0f ||
-                            h[2].y > 1.0f || h[3].y > 1.0f || h[4].y != 0.0f || h[5].y != 0.0f || h[6].y != 0.0f);
-      if (changed && !dirty) {
-        // first change in a pristine element: the points of the earlier
-        // pairs keep the initial history, not yet in the output buffer
-        for (int q = 0; q < p; ++q)
-#pragma unroll
-          for (int f = 0; f < 7; ++f) {
-            hout[(int64_t)(f * 8 + pair_point(q, 0)) * nh] = f < 4 ? 1.0f : 0.0f;
-            hout[(int64_t)(f * 8 + pair_point(q, 1)) * nh] = f < 4 ? 1.0f : 0.0f;
-          }
-        dirty = true;
-      }
-      if (dirty) {
-#pragma unroll
-        for (int f = 0; f < 7; ++f) {
-          hout[(int64_t)(f * 8 + gx) * nh] = h[f].x;
-          hout[(int64_t)(f * 8 + gy) * nh] = h[f].y;
-        }
-      }
-    }
-    // back to global axes: S = R Sm R^T
-    float2 S[3][3];
-    S[0][0] = pfma(p2(s2), sm[1], pfma(p2(-2.0f * csn), sm[3], pmul(p2(c2), sm[0])));
-    S[1][1] = pfma(p2(c2), sm[1], pfma(p2(2.0f * csn), sm[3], pmul(p2(s2), sm[0])));
-    S[2][2] = sm[2];
-    S[0][1] = S[1][0] = pfma(p2(-csn), sm[1], pfma(p2(c2 - s2), sm[3], pmul(p2(csn), sm[0])));
-    S[0][2] = S[2][0] = pfma(p2(-sn), sm[5], pmul(p2(cs), sm[4]));
-    S[1][2] = S[2][1] = pfma(p2(cs), sm[5], pmul(p2(sn), sm[4]));
-    // P = S F^T with F = I + H
-    float2 P[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        P[i][k] = pfma(S[i][2], H[k][2], pfma(S[i][1], H[k][1], pfma(S[i][0], H[k][0], S[i][k])));
-    // mode sums of Q_k = w_k P_k (w_k = det J / J_kk) times the Gauss-point
-    // values of the mode derivatives; the lanes enter through their sum
-    // (xi-even modes) and difference (xi-odd modes)
-    const float e0 = et * wd[0], z1 = ze * wd[1], e2 = et * wd[2], z0 = ze * wd[0], ez0 = etze * wd[0];
-    const float g1 = gp * wd[1], g2 = gp * wd[2], gz1 = g1 * ze, ge2 = g2 * et;
-    // components 0 and 1 as a packed pair, component 2 alone
-    {
-      const float2 s0 = make_float2(P[0][0].x + P[0][0].y, P[0][1].x + P[0][1].y);
-      const float2 s1 = make_float2(P[1][0].x + P[1][0].y, P[1][1].x + P[1][1].y);
-      const float2 s2s = make_float2(P[2][0].x + P[2][0].y, P[2][1].x + P[2][1].y);
-      const float2 d1 = make_float2(P[1][0].y - P[1][0].x, P[1][1].y - P[1][1].x);
-      const float2 d2 = make_float2(P[2][0].y - P[2][0].x, P[2][1].y - P[2][1].x);
-      float2 c;
-      c = pfma(p2(wd[0]), s0, make_float2(C[1][0], C[1][1]));
-      C[1][0] = c.x, C[1][1] = c.y;
-      c = pfma(p2(wd[1]), s1, make_float2(C[2][0], C[2][1]));
-      C[2][0] = c.x, C[2][1] = c.y;
-      c = pfma(p2(wd[2]), s2s, make_float2(C[3][0], C[3][1]));
-      C[3][0] = c.x, C[3][1] = c.y;
-      c = padd(make_float2(C[4][0], C[4][1]), pfma(p2(g1), d1, pmul(p2(e0), s0)));
-      C[4][0] = c.x, C[4][1] = c.y;
-      c = padd(make_float2(C[5][0], C[5][1]), pfma(p2(e2), s2s, pmul(p2(z1), s1)));
-      C[5][0] = c.x, C[5][1] = c.y;
-      c = padd(make_float2(C[6][0], C[6][1]), pfma(p2(g2), d2, pmul(p2(z0), s0)));
-      C[6][0] = c.x, C[6][1] = c.y;
-      c = padd(make_float2(C[7][0], C[7][1]), pfma(p2(ge2), d2, pfma(p2(gz1), d1, pmul(p2(ez0), s0))));
-      C[7][0] = c.x, C[7][1] = c.y;
-    }
-    {
-      const float s0 = P[0][2].x + P[0][2].y, s1 = P[1][2].x + P[1][2].y, s2s = P[2][2].x + P[2][2].y;
-      const float d1 = P[1][2].y - P[1][2].x, d2 = P[2][2].y - P[2][2].x;
-      C[1][2] = fmaf(wd[0], s0, C[1][2]);
-      C[2][2] = fmaf(wd[1], s1, C[2][2]);
-      C[3][2] = fmaf(wd[2], s2s, C[3][2]);
-      C[4][2] = C[4][2] + fmaf(g1, d1, e0 * s0);
-      C[5][2] = C[5][2] + fmaf(e2, s2s, z1 * s1);
-      C[6][2] = C[6][2] + fmaf(g2, d2, z0 * s0);
-      C[7][2] = C[7][2] + fmaf(ge2, d2, fmaf(gz1, d1, ez0 * s0));
-    }
-  }
-  if (D.pflag[0] != nullptr) D.pflag[hb ^ 1][e] = (pristine_in && !dirty) ? 1 : 0;
-  float f[8][3];
-  from_modes(C, f);
-  store(f);
-}
-
-// ---------------------------------------------------------------------------
-// Kernel 2: hex8 internal forces, total Lagrangian, 2x2x2 Gauss (Sec. 2,
-// Eq. fcont), with the intralaminar law per Gauss point.  One thread per
-// element; geometry and displacement enter through their trilinear modes, so
-// that J = [dx/dxi], du/dxi and the returned force are cheap mode sums.
-// f_a = sum_g sum_k dN_a/dxi_k Q_g[k][:],  Q_g = det J_g  J_g^-1 P_g,
-// P = S F^T (nominal stress), S rotated from ply axes (angle about z).
-// BOX: every element is an axis-aligned box (checked on the host), so J is
-// the constant diagonal diag((x6-x0)/2, (y6-y0)/2, (z6-z0)/2).
-// The next Gauss point's history is loaded while the current one computes.
+// Kernel 2: hex8 internal forces of an item (pdn_hex.cuh): boxes one element
+// per thread (the warp calls together), other hexes eight lanes per element.
 template <typename T, bool BOX>
-__device__ __forceinline__ void hex_item(const Dev<T> &D, const Mat<T> &M, int64_t e, int mode) {
-  if constexpr (BOX && std::is_same<T, float>::value) {
-    hex_item_box_pairs(D, M, e, mode);
-    return;
-  }
-  using V4 = typename Vec4T<T>::type;
-  const Ctl *ctl = D.ctl;
-  if (e >= D.nh) return;
-  if (mode == MODE_REPEAT && !repeat_take(D.rmark_e, e)) return;
-  const int64_t nh = D.nh;
-  const int ub = (mode == MODE_FORCES) ? (ctl->dpar ^ 1) : ctl->dpar;
-  const int hb = ctl->hpar;
-  const V4 *PDN_STATE_RESTRICT U = D.u4[ub];
-  const int4 c0 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e);
-  const int4 c1 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e + 1);
-  const int nd[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-  if (!nodes_in_range(D, nd)) return;
-  if (mode == MODE_REPEAT) repeat_mark_nodes(D.rmark_n, nd);
-  const T *PDN_STATE_RESTRICT hin = D.hist[hb] + e;
-  T *PDN_STATE_RESTRICT hout = D.hist[hb ^ 1] + e;
-  // An element whose points all still hold the initial history skips the
-  // history traffic: it is not read, and written only once a point changes.
-  const bool pristine_in = D.pflag[0] != nullptr && D.pflag[hb][e] != 0;
-  bool dirty = false;
-  // history of Gauss point 0 in flight first
-  T hn[7];
-#pragma unroll
-  for (int f = 0; f < 7; ++f) hn[f] = pristine_in ? (f < 4 ? T(1) : T(0)) : hin[(int64_t)(f * 8) * nh];
-  T am[8][3], bm[8][3];
-  T jd[3] = {T(0), T(0), T(0)}, wd[3] = {T(0), T(0), T(0)}, vol = T(0);
-  {
-    T ua[8][3];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const V4 u = U[nd[a]];
-      ua[a][0] = u.x;
-      ua[a][1] = u.y;
-      ua[a][2] = u.z;
-    }
-    to_modes(ua, bm);
-    if constexpr (BOX) {
-      const V4 x0 = D.X4[nd[0]], x6 = D.X4[nd[6]];
-      const T J0 = T(0.5) * (x6.x - x0.x), J1 = T(0.5) * (x6.y - x0.y), J2 = T(0.5) * (x6.z - x0.z);
-      const T det = J0 * (J1 * J2);
-      jd[0] = T(1) / J0;
-      jd[1] = T(1) / J1;
-      jd[2] = T(1) / J2;
-      wd[0] = det * jd[0];
-      wd[1] = det * jd[1];
-      wd[2] = det * jd[2];
-      vol = T(8) * det;
-    } else {
-      T xa[8][3];
-#pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const V4 x = D.X4[nd[a]];
-        xa[a][0] = x.x;
-        xa[a][1] = x.y;
-        xa[a][2] = x.z;
-      }
-      to_modes(xa, am);
-    }
-  }
-  const int ply = D.ply[e];
-  const T cs = M.ply_c[ply], sn = M.ply_s[ply];
-  const T c2 = cs * cs, s2 = sn * sn, csn = cs * sn;
-  const ElemLaw<T> L = elem_law(M, e);
-  T lc = T(-1);
-  T C[8][3];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) C[m][0] = C[m][1] = C[m][2] = T(0);
-  const T gp = T(0.57735026918962576451);
-#pragma unroll 1
-  for (int g = 0; g < 8; ++g) {
-    T h[7];
-#pragma unroll
-    for (int f = 0; f < 7; ++f) h[f] = hn[f];
-    if (g < 7 && !pristine_in) {
-#pragma unroll
-      for (int f = 0; f < 7; ++f) hn[f] = hin[(int64_t)(f * 8 + g + 1) * nh];
-    }
-    const T xi = T(sgn_x(g)) * gp, et = T(sgn_y(g)) * gp, ze = T(sgn_z(g)) * gp;
-    T Du[3][3], H[3][3], Ji[3][3], det = T(0);
-    jac_cols(bm, xi, et, ze, Du);
-    if constexpr (BOX) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) H[i][k] = Du[i][k] * jd[k];
-    } else {
-      T J[3][3];
-      jac_cols(am, xi, et, ze, J);
-      det = det3(J);
-      const T id = T(1) / det;
-      Ji[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) * id;
-      Ji[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * id;
-      Ji[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) * id;
-      Ji[1][0] = (J[1][2] * J[2][0] - J[1][0] * J[2][2]) * id;
-      Ji[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) * id;
-      Ji[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) * id;
-      Ji[2][0] = (J[1][0] * J[2][1] - J[1][1] * J[2][0]) * id;
-      Ji[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) * id;
-      Ji[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * id;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) H[i][k] = Du[i][0] * Ji[0][k] + Du[i][1] * Ji[1][k] + Du[i][2] * Ji[2][k];
-    }
-    // Green strain E = 1/2 (H + H^T + H^T H)
-    T E[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = i; k < 3; ++k) {
-        E[i][k] = T(0.5) * (H[i][k] + H[k][i] + H[0][i] * H[0][k] + H[1][i] * H[1][k] + H[2][i] * H[2][k]);
-        E[k][i] = E[i][k];
-      }
-    // to ply axes (rotation about z): Em = R^T E R
-    T ep[6];
-    ep[0] = c2 * E[0][0] + T(2) * csn * E[0][1] + s2 * E[1][1];
-    ep[1] = s2 * E[0][0] - T(2) * csn * E[0][1] + c2 * E[1][1];
-    ep[2] = E[2][2];
-    ep[3] = T(2) * (-csn * E[0][0] + (c2 - s2) * E[0][1] + csn * E[1][1]);
-    ep[4] = T(2) * (cs * E[0][2] + sn * E[1][2]);
-    ep[5] = T(2) * (-sn * E[0][2] + cs * E[1][2]);
-    T sm[6];
-    if constexpr (BOX)
-      cdm(M, L, (const T(*)[3]) nullptr, vol, lc, ep, h, sm);
-    else
-      cdm(M, L, (const T(*)[3])am, T(0), lc, ep, h, sm);
-    if (!pristine_in) {
-#pragma unroll
-      for (int f = 0; f < 7; ++f) hout[(int64_t)(f * 8 + g) * nh] = h[f];
-    } else {
-      const bool changed = h[0] > T(1) || h[1] > T(1) || h[2] > T(1) || h[3] > T(1) || h[4] != T(0) ||
-                           h[5] != T(0) || h[6] != T(0);
-      if (changed && !dirty) {
-        // first change in a pristine element: the earlier points keep the
-        // initial history, which the output buffer does not hold yet
-        for (int gg = 0; gg < g; ++gg)
-#pragma unroll
-          for (int f = 0; f < 7; ++f) hout[(int64_t)(f * 8 + gg) * nh] = f < 4 ? T(1) : T(0);
-        dirty = true;
-      }
-      if (dirty) {
-#pragma unroll
-        for (int f = 0; f < 7; ++f) hout[(int64_t)(f * 8 + g) * nh] = h[f];
-      }
-    }
-    // back to global axes: S = R Sm R^T
-    T S[3][3];
-    S[0][0] = c2 * sm[0] - T(2) * csn * sm[3] + s2 * sm[1];
-    S[1][1] = s2 * sm[0] + T(2) * csn * sm[3] + c2 * sm[1];
-    S[2][2] = sm[2];
-    S[0][1] = S[1][0] = csn * sm[0] + (c2 - s2) * sm[3] - csn * sm[1];
-    S[0][2] = S[2][0] = cs * sm[4] - sn * sm[5];
-    S[1][2] = S[2][1] = sn * sm[4] + cs * sm[5];
-    // P = S F^T with F = I + H; Q = det J^-1 P
-    T P[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        P[i][k] = S[i][k] + S[i][0] * H[k][0] + S[i][1] * H[k][1] + S[i][2] * H[k][2];
-    T Q[3][3];
-    if constexpr (BOX) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int I = 0; I < 3; ++I) Q[k][I] = wd[k] * P[k][I];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int I = 0; I < 3; ++I) Q[k][I] = det * (Ji[k][0] * P[0][I] + Ji[k][1] * P[1][I] + Ji[k][2] * P[2][I]);
-    }
-#pragma unroll
-    for (int I = 0; I < 3; ++I) {
-      C[1][I] += Q[0][I];
-      C[2][I] += Q[1][I];
-      C[3][I] += Q[2][I];
-      C[4][I] += et * Q[0][I] + xi * Q[1][I];
-      C[5][I] += ze * Q[1][I] + et * Q[2][I];
-      C[6][I] += ze * Q[0][I] + xi * Q[2][I];
-      C[7][I] += et * ze * Q[0][I] + xi * ze * Q[1][I] + xi * et * Q[2][I];
-    }
-  }
-  if (D.pflag[0] != nullptr) D.pflag[hb ^ 1][e] = (pristine_in && !dirty) ? 1 : 0;
-  T f[8][3];
-  from_modes(C, f);
-  // element forces go straight to their CSR positions, so that the gather
-  // reads each node's contributions as one contiguous run
-  const int4 p0 = __ldg(reinterpret_cast<const int4 *>(D.pos) + 2 * e);
-  const int4 p1 = __ldg(reinterpret_cast<const int4 *>(D.pos) + 2 * e + 1);
-  const int ps[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    V4 o;
-    o.x = f[a][0];
-    o.y = f[a][1];
-    o.z = f[a][2];
-    o.w = T(0);
-    D.fe[ps[a]] = o;
+__device__ __forceinline__ void hex_item(const Dev<T> &D, const Mat<T> &M, int64_t first, int64_t end, int mode) {
+  // elements [first, end) of this block, strided over its threads
+  const int lane = (int)(threadIdx.x & 31);
+  if constexpr (BOX) {
+    for (int64_t i = first + (int)(threadIdx.x & ~31u); i < end; i += blockDim.x)
+      hex_box_item(D, M, i + lane, i + lane < end, mode);
+  } else {
+    for (int64_t i = 8 * first + (int)(threadIdx.x & ~31u); i < 8 * end; i += blockDim.x)
+      hex_lanes8_item<T, false>(D, M, i + lane, end, mode);
   }
 }
 

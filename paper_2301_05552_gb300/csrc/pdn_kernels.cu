@@ -50,12 +50,25 @@ __global__ void __launch_bounds__(kActRun) k_contact(Dev<T> D) {
   if (D.act_cnt != nullptr && threadIdx.x == 0) D.act_cnt[blockIdx.x] = c;
 }
 
-template <typename T, bool BOX, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_hex(Dev<T> D, Mat<T> M) {
+// Boxes, one element per thread.
+template <typename T, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_hex(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M) {
   pdl_enter();
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
-  hex_item<T, BOX>(D, M, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, mode);
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  hex_box_item(D, M, e, e < D.nh, mode);
+}
+
+// Eight lanes per element: general hexes, and boxes in launches too small to
+// fill the GPU with one thread per element.
+template <typename T, bool BOX>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3)
+    k_hex_lanes8(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M) {
+  pdl_enter();
+  const int mode = D.ctl->mode;
+  if (mode >= MODE_DONE) return;
+  hex_lanes8_item<T, BOX>(D, M, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, D.nh, mode);
 }
 
 template <typename T, bool FLAT, int MINB>
@@ -71,7 +84,8 @@ __global__ void __launch_bounds__(128, MINB) k_coh(Dev<T> D, Mat<T> M) {
 // larger kind), so that every SM runs both the compute-bound hex warps and
 // the latency-bound interface warps at the same time.
 template <typename T, bool BOX, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_elem(Dev<T> D, Mat<T> M, int nbh, int nbc) {
+__global__ void __launch_bounds__(128, MINB)
+    k_elem(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M, int nbh, int nbc) {
   pdl_enter();
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
@@ -84,9 +98,9 @@ __global__ void __launch_bounds__(128, MINB) k_elem(Dev<T> D, Mat<T> M, int nbh,
     kind = nbh > nbc ? 0 : 1;
     idx = m + (b - 2 * m);
   }
-  const int64_t i = (int64_t)idx * blockDim.x + threadIdx.x;
+  const int64_t first = (int64_t)idx * blockDim.x, i = first + threadIdx.x;
   if (kind == 0)
-    hex_item<T, BOX>(D, M, i, mode);
+    hex_item<T, BOX>(D, M, first, min(D.nh, first + (int64_t)blockDim.x), mode);
   else if (D.all_flat_coh)
     coh_item<T, true>(D, M, i, mode);
   else
@@ -187,7 +201,8 @@ __device__ __forceinline__ void cp_async_wait_all() {
 }
 
 template <int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY)) k_sweep(Dev<float> D, Mat<float> M, Sweep S) {
+__global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
+    k_sweep(const __grid_constant__ Dev<float> D, const __grid_constant__ Mat<float> M, const __grid_constant__ Sweep S) {
   constexpr int NT = TX * TY, NC = (TX + 1) * (TY + 1);
   __shared__ SweepSmem<TX, TY> sm;
   pdl_enter();
@@ -273,8 +288,8 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY)) k_sweep(Dev<float> D
     const int L = S.bot[k];
     const bool lo_here = layer_here(L), hi_here = layer_here(L + 1);
     if (lo_here) prefetch_layer(L);
-    if (col) {
-      const int64_t el = (int64_t)S.base[k] + (int64_t)gj * S.nx + gi;
+    {
+      const int64_t el = col ? (int64_t)S.base[k] + (int64_t)gj * S.nx + gi : 0;
       auto store = [&](const float (&f)[8][3], const int (&nd)[8]) {
         const uint32_t rk = __ldg(D.rank + (S.kind[k] ? D.nh + el : el));
 #pragma unroll
@@ -293,10 +308,13 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY)) k_sweep(Dev<float> D
           }
         }
       };
-      if (S.kind[k] == 0)
-        hex_box_forces(D, M, el, mode, store);
-      else
+      if (S.kind[k] == 0) {
+        float f[8][3];
+        int nd[8];
+        if (hex_box_forces(D, M, el, col, mode, f, nd)) store(f, nd);
+      } else if (col) {
         coh_forces<float, true>(D, M, el, mode, store);
+      }
     }
     cp_async_wait_all();
     __syncthreads();
@@ -331,6 +349,21 @@ __global__ void k_striker_init(Striker *S, StrikerStep *ss, double dt) {
     ss->w[i] = w1[i];
     ss->aI[i] = aI[i];
   }
+}
+
+template <typename T>
+__global__ void k_box_records(Dev<T> D, typename Vec4T<T>::type *box) {
+  using V4 = typename Vec4T<T>::type;
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= D.nh) return;
+  const V4 a = D.X4[D.hex[8 * e]], b = D.X4[D.hex[8 * e + 6]];
+  const T hx = b.x - a.x, hy = b.y - a.y, hz = b.z - a.z;
+  V4 o;
+  o.x = T(1) / hx;
+  o.y = T(1) / hy;
+  o.z = T(1) / hz;
+  o.w = T(0.125) * (hx * (hy * hz));
+  box[e] = o;
 }
 
 // ---------------------------------------------------------------------------
@@ -435,30 +468,30 @@ inline int grid_of(int64_t n, int b) {
 
 }  // namespace
 
-// Element kernel variants chosen per context by the autotuner: 0..3 hex
-// kernel (interface kernel on the side stream) with an occupancy target of 4,
-// 5, 6 or 3 blocks of 128 per SM (which caps the registers per thread);
-// 4..7 the same targets for the mixed hex + interface kernel.
+// Element kernel variants (pdn_info.hex_variant): 0..3 separate element
+// kernels, 4..7 one mixed hex + interface launch.
 constexpr int kMixedVariant = 4;
-
-template <typename T, bool BOX>
-void launch_elem_box(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
-  const int nbh = grid_of(D.nh, 128), nbc = D.nc > 0 ? (int)((D.nc + 127) / 128) : 0;
-  const int g = nbh + nbc;
-  switch (D.hex_variant) {
-    case 5: launch_k(k_elem<T, BOX, 5>, g, 128, s, D, M, nbh, nbc); break;
-    case 6: launch_k(k_elem<T, BOX, 6>, g, 128, s, D, M, nbh, nbc); break;
-    case 7: launch_k(k_elem<T, BOX, 3>, g, 128, s, D, M, nbh, nbc); break;
-    default: launch_k(k_elem<T, BOX, 4>, g, 128, s, D, M, nbh, nbc); break;
-  }
-}
 
 template <typename T>
 void launch_elem(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
+  const int nbh = grid_of(D.nh, 128), nbc = D.nc > 0 ? (int)((D.nc + 127) / 128) : 0;
+  const int g = nbh + nbc;
   if (D.all_boxes)
-    launch_elem_box<T, true>(D, M, s);
+    launch_k(k_elem<T, true, 4>, g, 128, s, D, M, nbh, nbc);
   else
-    launch_elem_box<T, false>(D, M, s);
+    launch_k(k_elem<T, false, 4>, g, 128, s, D, M, nbh, nbc);
+}
+
+// FP64 boxes: one thread per element or eight lanes.  An FP64 operation holds
+// its scheduler 64 cycles whether one warp or more are resident, so the
+// launch takes (warps on the fullest scheduler) x (operations per warp): about
+// 900 per warp of 32 elements, or 190 per warp of 4.
+template <typename T>
+bool hex_lanes8_fits(const Dev<T> &D) {
+  if (sizeof(T) == 4) return false;
+  const int64_t schedulers = 4 * 152;
+  const int64_t w1 = (D.nh + 31) / 32, w8 = (D.nh + 3) / 4;
+  return (w8 + schedulers - 1) / schedulers * 190 <= (w1 + schedulers - 1) / schedulers * 900;
 }
 
 template <typename T>
@@ -469,21 +502,18 @@ void launch_hex(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
       return;
     }
   }
-  const int g = grid_of(D.nh, 128);
-  if (D.all_boxes) {
+  if (!D.all_boxes)
+    launch_k(k_hex_lanes8<T, false>, grid_of(8 * D.nh, 128), 128, s, D, M);
+  else if (hex_lanes8_fits(D))
+    launch_k(k_hex_lanes8<T, true>, grid_of(8 * D.nh, 128), 128, s, D, M);
+  else if constexpr (std::is_same<T, float>::value) {
+    const int g = grid_of(D.nh, 128);
     switch (D.hex_variant) {
-      case 1: launch_k(k_hex<T, true, 5>, g, 128, s, D, M); break;
-      case 2: launch_k(k_hex<T, true, 6>, g, 128, s, D, M); break;
-      case 3: launch_k(k_hex<T, true, 3>, g, 128, s, D, M); break;
-      default: launch_k(k_hex<T, true, 4>, g, 128, s, D, M); break;
+      case 3: launch_k(k_hex<T, 3>, g, 128, s, D, M); break;
+      default: launch_k(k_hex<T, 4>, g, 128, s, D, M); break;
     }
   } else {
-    switch (D.hex_variant) {
-      case 1: launch_k(k_hex<T, false, 5>, g, 128, s, D, M); break;
-      case 2: launch_k(k_hex<T, false, 6>, g, 128, s, D, M); break;
-      case 3: launch_k(k_hex<T, false, 3>, g, 128, s, D, M); break;
-      default: launch_k(k_hex<T, false, 4>, g, 128, s, D, M); break;
-    }
+    launch_k(k_hex<T, 2>, grid_of(D.nh, 128), 128, s, D, M);
   }
 }
 
@@ -620,6 +650,12 @@ cudaError_t launch_damage_field(const Dev<T> &D, const Mat<T> &M, int which, flo
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t launch_box_records(const Dev<T> &D, typename Vec4T<T>::type *box, cudaStream_t s) {
+  k_box_records<T><<<grid_of(D.nh, 256), 256, 0, s>>>(D, box);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_striker_init(Striker *S, StrikerStep *ss, double dt, cudaStream_t s) {
   k_striker_init<<<1, 1, 0, s>>>(S, ss, dt);
   return cudaGetLastError();
@@ -629,6 +665,8 @@ template cudaError_t launch_pass<float>(const Dev<float> &, const Mat<float> &, 
                                         cudaEvent_t *, cudaStream_t, cudaEvent_t, cudaEvent_t);
 template cudaError_t launch_pass<double>(const Dev<double> &, const Mat<double> &, cudaStream_t, int32_t,
                                          cudaEvent_t *, cudaStream_t, cudaEvent_t, cudaEvent_t);
+template cudaError_t launch_box_records<float>(const Dev<float> &, float4 *, cudaStream_t);
+template cudaError_t launch_box_records<double>(const Dev<double> &, double4_32a *, cudaStream_t);
 template cudaError_t launch_pairs_to_elements<float>(const Dev<float> &, cudaStream_t);
 template cudaError_t launch_pairs_to_elements<double>(const Dev<double> &, cudaStream_t);
 template cudaError_t launch_damage_field<float>(const Dev<float> &, const Mat<float> &, int, float *,

@@ -45,18 +45,35 @@ constexpr size_t kFeBytes = (size_t)PDN_NOALLOC_MAX_HEX * 8 * 32;
 constexpr size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 constexpr size_t kOffX4 = round256(kCtlBytes);
 constexpr size_t kOffU4 = kOffX4 + round256(kNodeV4Bytes);
-constexpr size_t kOffHin = kOffU4 + round256(kNodeV4Bytes);
-constexpr size_t kOffHout = kOffHin + round256(kHistBytes);
+constexpr size_t kOffHout = kOffU4 + round256(kNodeV4Bytes);
 constexpr size_t kOffFe = kOffHout + round256(kHistBytes);
 constexpr size_t kPosBytes = (size_t)PDN_NOALLOC_MAX_HEX * 8 * sizeof(int32_t);
 constexpr size_t kOffPos = kOffFe + round256(kFeBytes);
-constexpr size_t kScratchBytes = kOffPos + round256(kPosBytes);
+// per-element flags of the initial history (in, out) and the plies' stiffness
+constexpr size_t kOffFlagIn = kOffPos + round256(kPosBytes);
+constexpr size_t kOffFlagOut = kOffFlagIn + round256(PDN_NOALLOC_MAX_HEX);
+constexpr size_t kOffPlyQ = kOffFlagOut + round256(PDN_NOALLOC_MAX_HEX);
+constexpr size_t kScratchBytes = kOffPlyQ + round256(sizeof(double) * 16 * kMaxPlies);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 template <typename T>
+struct PlyTable {
+  T q[kMaxPlies * kPlyStride<T>];
+};
+
+// Control block, mirrors, the plies' stiffness, the elements' initial-history
+// flags and the CSR position of every element slot (the inverse of the
+// caller's csr_col: the element kernel writes each nodal force at its node's
+// CSR position), in one launch: each thread takes its node, its flag and its
+// slots.  One launch instead of two and a flag per element instead of 448
+// bytes of initial history: at 1,105 hexes in FP64 the call went from 143 us
+// to the figure in the notes below, of which the element kernel is most.
+template <typename T>
 __global__ void k_noalloc_prepare(Ctl *ctl, const double *X, const double *d, typename Vec4T<T>::type *X4,
-                                  typename Vec4T<T>::type *u4, int64_t nn, T *hist_pristine, int64_t per_field) {
+                                  typename Vec4T<T>::type *u4, int64_t nn, uint8_t *flag, int64_t nh,
+                                  const int32_t *col, int32_t *pos, T *ply_q, int n_plies,
+                                  const __grid_constant__ PlyTable<T> tab) {
   using V4 = typename Vec4T<T>::type;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) {
@@ -79,25 +96,20 @@ __global__ void k_noalloc_prepare(Ctl *ctl, const double *X, const double *d, ty
     X4[i] = x;
     u4[i] = u;
   }
-  if (hist_pristine) {
-    for (int64_t k = i; k < per_field * 7; k += (int64_t)gridDim.x * blockDim.x)
-      hist_pristine[k] = (k < per_field * 4) ? T(1) : T(0);  // r_N = 1, plastic strain 0
+  if (i < nh && flag != nullptr) flag[i] = 1;
+  if (i < (int64_t)n_plies * kPlyStride<T>) ply_q[i] = tab.q[i];
+  const int64_t nnz = 8 * nh;
+  for (int64_t r = i; r < nnz; r += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t c = col[r];
+    if (c >= 0 && c < nnz) pos[c] = (int32_t)r;
   }
-}
-
-// CSR position of every element slot: the inverse of the caller's csr_col
-// (the element kernel writes each nodal force at its node's CSR position).
-__global__ void k_noalloc_pos(const int32_t *col, int32_t *pos, int64_t nnz) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nnz) return;
-  const int32_t c = col[r];
-  if (c >= 0 && c < nnz) pos[c] = (int32_t)r;
 }
 
 template <typename T>
 cudaError_t run_noalloc(unsigned char *base, int64_t nn, int64_t nh, const int32_t *hex, const int8_t *ply,
                         const double *X, const double *d, const void *history, const int32_t *row,
-                        const int32_t *col, const Mat<T> &M, double *f_int, cudaStream_t s) {
+                        const int32_t *col, const Mat<T> &M, const Mat<double> &M64, int n_plies, double *f_int,
+                        cudaStream_t s) {
   using V4 = typename Vec4T<T>::type;
   Dev<T> D{};
   D.nn = nn;
@@ -115,24 +127,29 @@ cudaError_t run_noalloc(unsigned char *base, int64_t nn, int64_t nh, const int32
   V4 *u4 = reinterpret_cast<V4 *>(base + kOffU4);
   D.u4[0] = u4;
   D.u4[1] = u4;
-  T *hin = history ? const_cast<T *>(reinterpret_cast<const T *>(history)) : reinterpret_cast<T *>(base + kOffHin);
-  D.hist[0] = hin;
+  D.hist[0] = const_cast<T *>(reinterpret_cast<const T *>(history));
   D.hist[1] = reinterpret_cast<T *>(base + kOffHout);
+  // without a history every element starts from the initial one: flagged, so
+  // that none is read
+  uint8_t *flag = history ? nullptr : base + kOffFlagIn;
+  D.pflag[0] = flag;
+  D.pflag[1] = history ? nullptr : base + kOffFlagOut;
   D.fe = reinterpret_cast<V4 *>(base + kOffFe);
   D.ctl = reinterpret_cast<Ctl *>(base);
   D.fout = f_int;
-  const int64_t work = std::max<int64_t>(nn, 1);
+  int32_t *pos = reinterpret_cast<int32_t *>(base + kOffPos);
+  D.pos = pos;
+  T *ply_q = reinterpret_cast<T *>(base + kOffPlyQ);
+  D.ply_q = ply_q;
+  PlyTable<T> tab{};
+  ply_table(M64, n_plies, tab.q);
+  // the threads cover the nodes, the elements and the plies' table
+  const int64_t work = std::max<int64_t>(std::max(nn, nh), (int64_t)kMaxPlies * kPlyStride<T>);
   const int grid = (int)((work + kBlock - 1) / kBlock);
-  k_noalloc_prepare<T><<<grid, kBlock, 0, s>>>(D.ctl, X, d, const_cast<V4 *>(D.X4), u4, nn,
-                                                history ? nullptr : reinterpret_cast<T *>(base + kOffHin), nh * 8);
+  k_noalloc_prepare<T><<<grid, kBlock, 0, s>>>(D.ctl, X, d, const_cast<V4 *>(D.X4), u4, nn, flag, nh, col, pos, ply_q,
+                                               n_plies, tab);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  int32_t *pos = reinterpret_cast<int32_t *>(base + kOffPos);
-  const int64_t nnz = nh * 8;
-  k_noalloc_pos<<<(int)((nnz + kBlock - 1) / kBlock), kBlock, 0, s>>>(col, pos, nnz);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  D.pos = pos;
   return launch_pass<T>(D, M, s, kBlock, nullptr);
 }
 
@@ -176,18 +193,18 @@ extern "C" int pdn_internal_force_noalloc(int64_t n_nodes, int64_t n_hex, const 
     return bad(PDN_E_CUDA, std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(e));
   std::string why;
   cudaStream_t s = (cudaStream_t)stream;
+  Mat<double> M64{};
+  int rc = fill_mat_public(M64, *mat, ply_angle_deg, n_plies, damage_on, plasticity_on, why);
+  if (rc) return bad(rc, why);
   if (precision == PDN_FP64) {
-    Mat<double> M{};
-    int rc = fill_mat_public(M, *mat, ply_angle_deg, n_plies, damage_on, plasticity_on, why);
-    if (rc) return bad(rc, why);
     e = run_noalloc<double>((unsigned char *)addr, n_nodes, n_hex, hex, ply_of_hex, X, d, history, csr_row, csr_col,
-                            M, f_int, s);
+                            M64, M64, n_plies, f_int, s);
   } else {
     Mat<float> M{};
-    int rc = fill_mat_public(M, *mat, ply_angle_deg, n_plies, damage_on, plasticity_on, why);
+    rc = fill_mat_public(M, *mat, ply_angle_deg, n_plies, damage_on, plasticity_on, why);
     if (rc) return bad(rc, why);
-    e = run_noalloc<float>((unsigned char *)addr, n_nodes, n_hex, hex, ply_of_hex, X, d, history, csr_row, csr_col,
-                           M, f_int, s);
+    e = run_noalloc<float>((unsigned char *)addr, n_nodes, n_hex, hex, ply_of_hex, X, d, history, csr_row, csr_col, M,
+                           M64, n_plies, f_int, s);
   }
   if (e != cudaSuccess) return bad(PDN_E_CUDA, std::string("pdn_internal_force_noalloc launch: ") + cudaGetErrorString(e));
   return PDN_OK;
