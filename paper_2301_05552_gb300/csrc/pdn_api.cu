@@ -970,6 +970,33 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
       std::vector<char>().swap(iw);
     }
   }
+  // Force planes instead of slots (FP32, eight slots per node, no column
+  // sweep) where three quarters of the hexes have each corner one node id
+  // after their predecessor's, as in a structured numbering (every element of
+  // a row but its first): a warp's stores to a plane are then whole lines.
+  // Otherwise each would be 32 separate 4-byte stores, three times the
+  // 16-byte ones of the slots.  PDN_PLANES=0, read here, keeps the slots.
+  const char *pl = std::getenv("PDN_PLANES");
+  bool planes = opt->precision == PDN_FP32_FORCE && ell && !sweep_on && !(pl && pl[0] == '0' && pl[1] == '\0');
+  if (planes) {
+    std::vector<int64_t> next_t(n_threads, 0);
+    parallel_chunks(nh, [&](int64_t b, int64_t e1, int t) {
+      int64_t n = 0;
+      for (int64_t e = std::max<int64_t>(b, 1); e < e1; ++e) {
+        const int32_t *p = mesh->hex + (e - 1) * 8, *q = p + 8;
+        int same = 0;
+        for (int a = 0; a < 8; ++a) same += q[a] == p[a] + 1;
+        n += same == 8;
+      }
+      next_t[t] += n;
+    });
+    int64_t n = 0;
+    for (int t = 0; t < n_threads; ++t) n += next_t[t];
+    planes = 4 * n >= 3 * nh;
+    if (planes) slot_compact = false;
+  }
+  const int64_t plane_n = (nn + 31) & ~int64_t(31);
+  const size_t fe_bytes = planes ? sizeof(float) * 24 * plane_n : (opt->precision == PDN_FP64 ? 8 : 4) * 4 * n_slots;
   // interface stable step: rho_bar = rho * h, h = volume / face area of the
   // thinner hex sharing a face with the interface element
   double dtc = INFINITY;
@@ -1067,7 +1094,7 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
       P.pflag[b] = A.take<uint8_t>((nh + 15) & ~int64_t(15));
       P.cflag[b] = A.take<uint8_t>(nc1);
     }
-    P.fe = A.take<char>(ts * 4 * n_slots);
+    P.fe = A.take<char>(fe_bytes);
     P.rel = A.take<uint8_t>(ns1);
     P.act_cnt = A.take<int32_t>(sizeof(int32_t) * ((ns1 + kActRun - 1) / kActRun));
     P.rmark_e = A.take<uint8_t>(nh + nc);
@@ -1199,7 +1226,7 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
       k_fill_hist_float<<<grid_of(nh * 8 * 7, 256), 256>>>(reinterpret_cast<float *>(d_hist[b]), nh * 8, 4);
     chk(cudaGetLastError());
   }
-  chk(cudaMemset(d_fe, 0, ts * 4 * n_slots));  // the padding slots stay zero
+  chk(cudaMemset(d_fe, 0, fe_bytes));  // the padding slots stay zero
   chk(cudaMemset(d_rel, 0, std::max<int64_t>(ns, 1)));
   chk(cudaMemset(d_rmark_e, 0, nh + nc));
   chk(cudaMemset(d_rmark_n, 0, nn));
@@ -1257,7 +1284,9 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
       D.pflag[b] = P.pflag[b];
       D.cflag[b] = P.cflag[b];
     }
-    D.fe = reinterpret_cast<V4 *>(d_fe);
+    D.fe = planes ? nullptr : reinterpret_cast<V4 *>(d_fe);
+    D.fplane = planes ? reinterpret_cast<float *>(d_fe) : nullptr;
+    D.fplane_n = plane_n;
     D.rel = d_rel;
     D.act_cnt = P.act_cnt;
     // PDN_FULL_REPEAT=1: repeated passes evaluate every element and node

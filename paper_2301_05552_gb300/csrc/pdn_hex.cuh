@@ -301,6 +301,12 @@ __device__ __forceinline__ void hex_lanes8_item(const Dev<T> &D, const Mat<T> &M
   const LaneForce<T> r = hex_lanes8<T, BOX>(D, M, e, valid, mode);
   if (!valid) return;
   if (mode == MODE_REPEAT && D.rmark_n != nullptr) D.rmark_n[r.nd] = 1;
+  if constexpr (sizeof(T) == 4) {
+    if (D.fplane != nullptr) {
+      plane_store(D.fplane, D.fplane_n, (int)((__ldg(D.rank + e) >> (3 * r.a)) & 7u), r.nd, r.f[0], r.f[1], r.f[2]);
+      return;
+    }
+  }
   V4 o;
   o.x = r.f[0];
   o.y = r.f[1];
@@ -763,6 +769,12 @@ __device__ __forceinline__ void hex_box_item(const Dev<T> &D, const Mat<T> &M, i
   T f[8][3];
   int nd[8];
   if (!hex_box_forces(D, M, e, valid, mode, f, nd)) return;
+  if constexpr (sizeof(T) == 4) {
+    if (D.fplane != nullptr) {
+      plane_store8(D, D.hex, e, e, f);
+      return;
+    }
+  }
   const uint32_t rk = D.rank != nullptr ? __ldg(D.rank + e) : 0u;
   int ps[8];
   element_slots(D, D.hex, e, reinterpret_cast<const int4 *>(D.pos) + 2 * e, rk, ps);

@@ -179,6 +179,11 @@ struct Dev {
   uint8_t *pflag[2];       // [nh]
   uint8_t *cflag[2];       // [nc]
   V4 *fe;                  // [(nh + nc) * 8] element nodal forces
+  // FP32 element forces as planes: component i of the slot of rank r of node j
+  // at fplane[(3 r + i) fplane_n + j] (fplane_n: nn rounded up to 32); fe is
+  // then not used.  Null: slots of fe.
+  float *fplane;
+  int64_t fplane_n;
   // contact
   uint8_t *act[2];         // [ns] contact set by step parity
   uint8_t *rel;            // [ns] released in the current step

@@ -320,6 +320,12 @@ __device__ __forceinline__ void coh_item(const Dev<T> &D, const Mat<T> &M, int64
   if (c >= D.nc) return;
   const uint32_t rk = D.rank != nullptr ? __ldg(D.rank + D.nh + c) : 0u;
   coh_forces<T, FLAT>(D, M, c, mode, [&](const T (&f)[8][3], const int (&nd)[8]) {
+    if constexpr (sizeof(T) == 4) {
+      if (D.fplane != nullptr) {
+        plane_store8(D, D.coh, c, D.nh + c, f);
+        return;
+      }
+    }
     int ps[8];
     element_slots(D, D.coh, c, reinterpret_cast<const int4 *>(D.pos) + 2 * (D.nh + c), rk, ps);
 #pragma unroll
@@ -819,8 +825,7 @@ __device__ __forceinline__ void gather_item(const Dev<T> &D, int64_t j, int mode
     // the node state above
     const V4 *fs = D.fe + 8 * j;
     V4 f[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f[k] = fs[k];
+    load_slots<0, 8>(D, fs, j, f);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       fx += f[k].x;
@@ -928,12 +933,9 @@ __device__ __forceinline__ void gather_pair_item(const Dev<T> &D, const Mat<T> &
   const int2 ip = D.ipair[j];
   const V4 *fs = D.fe + 8 * j;
   V4 f[8];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) f[k] = fs[k];
+  load_slots<0, 4>(D, fs, j, f);
   const int nhx = (ip.y >> 4) & 15;
-#pragma unroll
-  for (int k = 4; k < 8; ++k)
-    if (k < nhx) f[k] = fs[k];
+  if (nhx > 4) load_slots<4, 8>(D, fs, j, f);
   T fx = T(0), fy = T(0), fz = T(0);
 #pragma unroll
   for (int k = 0; k < 8; ++k)
@@ -982,12 +984,8 @@ __device__ __forceinline__ void gather_pair_layered_item(const Dev<T> &D, const 
   const int64_t pj = upper ? j - (int64_t)L : j + (int64_t)L;
   const V4 *fs = D.fe + (D.slot_compact ? compact_slot_base(D, lay, j) : 8 * j);
   V4 f[8];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) f[k] = fs[k];
-  if (!pair) {
-#pragma unroll
-    for (int k = 4; k < 8; ++k) f[k] = fs[k];
-  }
+  load_slots<0, 4>(D, fs, j, f);
+  if (!pair) load_slots<4, 8>(D, fs, j, f);
   V4 u;
   T rin = T(0);
   if (pair) {

@@ -767,6 +767,10 @@ __global__ void __launch_bounds__(kHexSurBlock, 3) k_hex_sur(Dev<float> D, Mat<f
   if (D.pflag[0] != nullptr) D.pflag[hb ^ 1][el] = (pristine_in && !dirty) ? 1 : 0;
   float f[8][3];
   from_modes(C, f);
+  if (D.fplane != nullptr) {
+    plane_store8(D, D.hex, el, el, f);
+    return;
+  }
   int ps[8];
   element_slots(D, D.hex, el, reinterpret_cast<const int4 *>(D.pos) + 2 * el,
                 D.rank != nullptr ? __ldg(D.rank + el) : 0u, ps);
