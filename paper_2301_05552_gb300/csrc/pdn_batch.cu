@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kBatchBlock, MINB) k_batch(BatchArgs<T> A) {
         switch (tl.y) {
           case TK_CONTACT:
             if (mode == MODE_ADVANCE || mode == MODE_REPEAT)
-              for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) contact_item(sD, i, mode);
+              for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) contact_item(sD, i, mode, contact_node(sD, i));
             break;
           case TK_HEX:
             if (mode < MODE_DONE) {
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kBatchBlock, MINB) k_batch_flow(FlowArgs<T> A)
     switch (tl.y) {
       case TK_CONTACT:
         if (mode == MODE_ADVANCE || mode == MODE_REPEAT)
-          for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) contact_item(sD, i, mode);
+          for (int64_t i = tl.z + threadIdx.x; i < tl.w; i += blockDim.x) contact_item(sD, i, mode, contact_node(sD, i));
         break;
       case TK_HEX:
         if (mode < MODE_DONE) {

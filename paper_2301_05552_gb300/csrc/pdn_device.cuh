@@ -561,26 +561,22 @@ __device__ __forceinline__ void czm(const Mat<T> &M, const T (&dl)[3], T rin, T 
 }
 
 
-__device__ __forceinline__ void striker_rk4(const Striker &S, double dt, double (&c1)[3],
-                                            double (&w1)[3], double (&aI)[3]) {
-  double ga[3];
-  const double iM = S.iM;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) ga[i] = S.g[i] - S.F[i] * iM;
-  const double an = ga[0] * S.axis[0] + ga[1] * S.axis[1] + ga[2] * S.axis[2];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    aI[i] = an * S.axis[i];
-    const double k1c = dt * S.w[i], k1w = dt * aI[i];
-    const double k2c = dt * (S.w[i] + 0.5 * k1w), k2w = dt * aI[i];
-    const double k3c = dt * (S.w[i] + 0.5 * k2w), k3w = dt * aI[i];
-    const double k4c = dt * (S.w[i] + k3w), k4w = dt * aI[i];
-    // weights 1/6, 1/3, 1/3, 1/6 as products (FP64 division is a long
-    // dependent sequence on this part and this runs on the critical path)
-    constexpr double s6 = 1.0 / 6.0, s3 = 1.0 / 3.0;
-    c1[i] = S.c[i] + k1c * s6 + k2c * s3 + k3c * s3 + k4c * s6;
-    w1[i] = S.w[i] + k1w * s6 + k2w * s3 + k3w * s3 + k4w * s6;
-  }
+// Striker of the next step (Eq. rk4): the acceleration along the impact
+// direction is held over the step.  Component i from its acceleration aI.
+__device__ __forceinline__ void striker_rk4(double c, double w, double aI, double dt, double &c1, double &w1) {
+  const double k1c = dt * w, k1w = dt * aI;
+  const double k2c = dt * (w + 0.5 * k1w), k2w = dt * aI;
+  const double k3c = dt * (w + 0.5 * k2w), k3w = dt * aI;
+  const double k4c = dt * (w + k3w), k4w = dt * aI;
+  // weights 1/6, 1/3, 1/3, 1/6 as products (FP64 division is a long
+  // dependent sequence on this part and this runs on the critical path)
+  constexpr double s6 = 1.0 / 6.0, s3 = 1.0 / 3.0;
+  c1 = c + k1c * s6 + k2c * s3 + k3c * s3 + k4c * s6;
+  w1 = w + k1w * s6 + k2w * s3 + k3w * s3 + k4w * s6;
+}
+// Acceleration along the impact direction from that of the free striker.
+__device__ __forceinline__ double striker_along(double g0, double g1, double g2, const double (&axis)[3]) {
+  return g0 * axis[0] + g1 * axis[1] + g2 * axis[2];
 }
 
 }  // namespace detail

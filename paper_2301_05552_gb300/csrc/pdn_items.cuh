@@ -38,15 +38,40 @@ namespace detail {
 // step, Eq. rk4) was produced by the tail of the previous pass, or by
 // k_striker_init after pdn_set_impactor; this kernel only reads it.
 // Returns whether node s is in the contact set when the item is done.
+//
+// The kernel is a chain of memory latencies (a few microseconds for 10^4
+// nodes, of which some tens compute anything), so the loads come in as few
+// rounds as their addresses allow: what no pass writes (ContactNode) before
+// the wait on the previous kernel, then everything the screen reads, then the
+// state of the nodes near the striker.  With the screen's loads behind each
+// other's branches there were two rounds more.
 template <typename T>
-__device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mode) {
+struct ContactNode {
+  int64_t j;
+  typename Vec4T<T>::type x;
+  uint8_t fl;
+};
+template <typename T>
+__device__ __forceinline__ ContactNode<T> contact_node(const Dev<T> &D, int64_t s) {
+  ContactNode<T> q{};
+  if (s >= D.ns) return q;
+  q.j = D.surf_base >= 0 ? D.surf_base + s : D.surf[s];
+#ifdef PDN_CHECK
+  if (q.j < 0 || q.j >= D.nn) return q;  // contact_item records it
+#endif
+  q.x = D.X4[q.j];
+  q.fl = D.nflag[q.j];
+  return q;
+}
+template <typename T>
+__device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mode, const ContactNode<T> &q) {
   using V4 = typename Vec4T<T>::type;
   const Ctl *ctl = D.ctl;
   if (s >= D.ns) return false;
   const Striker *S = D.imp;
   const StrikerStep *ss = D.imp_step;
   const int64_t nn = D.nn, ns = D.ns;
-  const int64_t j = D.surf_base >= 0 ? D.surf_base + s : D.surf[s];
+  const int64_t j = q.j;
 #ifdef PDN_CHECK
   if (j < 0 || j >= D.nn) {
     atomicCAS(&D.ctl->check, 0, (int32_t)CHECK_SURFACE_NODE);
@@ -58,25 +83,23 @@ __device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mod
   double *d = D.d[cur];
   double *v = D.v[cur];
   if (mode == MODE_ADVANCE) {
-    D.rel[s] = 0;
-    uint8_t a = 0;
-    const uint8_t fl = D.nflag[j];
+    const uint8_t fl = q.fl;
+    const V4 xr = q.x;
     const bool was_active = D.act[ppar][s] != 0;
-    bool near = was_active;
-    if (!near && S->has && (fl & 7) != 7) {
-      // FP32 prefilter: nodes farther than R + 0.05 mm from the centre cannot
-      // be in contact (the FP32 distance error here is below 1e-4 mm); only
-      // the others take the FP64 gap test below.
-      const V4 xr = D.X4[j];
-      const V4 ur = D.u4[cur][j];
-      const float dx = (float)xr.x + (float)ur.x - (float)ss->c[0];
-      const float dy = (float)xr.y + (float)ur.y - (float)ss->c[1];
-      const float dz = (float)xr.z + (float)ur.z - (float)ss->c[2];
-      const float mag = fabsf((float)xr.x) + fabsf((float)xr.y) + fabsf((float)xr.z);
-      const float rr = (float)S->R + 0.05f + 4e-6f * mag;
-      near = dx * dx + dy * dy + dz * dz < rr * rr;
-    }
-    if (near && S->has && (fl & 7) != 7) {
+    const V4 ur = D.u4[cur][j];
+    const bool can = S->has && (fl & 7) != 7;
+    // FP32 prefilter: nodes farther than R + 0.05 mm from the centre cannot
+    // be in contact (the FP32 distance error here is below 1e-4 mm); only
+    // the others take the FP64 gap test below.
+    const float dx = (float)xr.x + (float)ur.x - (float)ss->c[0];
+    const float dy = (float)xr.y + (float)ur.y - (float)ss->c[1];
+    const float dz = (float)xr.z + (float)ur.z - (float)ss->c[2];
+    const float mag = fabsf((float)xr.x) + fabsf((float)xr.y) + fabsf((float)xr.z);
+    const float rr = (float)S->R + 0.05f + 4e-6f * mag;
+    const bool near = was_active || dx * dx + dy * dy + dz * dz < rr * rr;
+    uint8_t a = 0;
+    D.rel[s] = 0;
+    if (near && can) {
       // every load of the node and the striker is issued before the first
       // store (a store to the trial copy could alias them otherwise)
       double x[3], r2 = 0.0, dj[3], vj[3], w[3];
@@ -365,22 +388,31 @@ __device__ __forceinline__ uint32_t flag_mask16(uint4 q) {
 template <typename T, bool RUNS = false>
 __device__ void tail_block(const Dev<T> &D, int mode) {
   Ctl *ctl = D.ctl;
-  // the control block and the striker are read once, early, into registers;
+  // Warp 0 takes the decision: the control block, the striker and the pass's
+  // non-finite flag (raised by the gather, which has completed) are read once,
+  // early, into its registers, so that their latency overlaps the reduction;
   // the striker only by passes that can commit a step (an internal-force
-  // evaluation may have no striker at all: D.imp is then null)
+  // evaluation may have no striker at all: D.imp is then null).  Component i
+  // of the striker's vectors is lane i's: an FP64 instruction holds its
+  // scheduler 64 cycles whatever its active lanes, and one thread's commit
+  // and striker update were 82 of them (2.7 us of this kernel), now 32.
   const bool stepping = (mode == MODE_ADVANCE || mode == MODE_REPEAT);
+  const int lane0 = (int)threadIdx.x & 31, comp = lane0 < 2 ? lane0 : 2;
   Ctl c;
-  Striker S;
-  StrikerStep ss;
+  double axis[3] = {0.0, 0.0, 0.0}, s_iM = 0.0, s_g = 0.0, n_c = 0.0, n_w = 0.0;
   int nf = 0;
-  if (threadIdx.x == 0) {
-    // the pass's non-finite flag (raised by the gather, which has completed)
-    // is read here, early, so that its latency overlaps the reduction
+  if (threadIdx.x < 32) {
     nf = *(volatile int *)&ctl->nonfinite;
     c = *ctl;
     if (stepping) {
-      S = *D.imp;
-      ss = *D.imp_step;
+      const Striker *S = D.imp;
+      const StrikerStep *ss = D.imp_step;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) axis[i] = S->axis[i];
+      s_iM = S->iM;
+      s_g = S->g[comp];
+      n_c = ss->c[comp];
+      n_w = ss->w[comp];
     }
   }
   // Reaction sum over the active contact nodes in a fixed order that does
@@ -596,38 +628,35 @@ __device__ void tail_block(const Dev<T> &D, int mode) {
         }
       }
     }
+    // Sums over the warp by xor-shuffles 16, 8, 4, 2, 1.  The first two rounds
+    // also part the components (lanes 0-7 keep x, 8-15 y, 16-23 z), so that six
+    // FP64 additions do what fifteen did; every sum has the same tree.
+    double fs = 0.0;
     if (__any_sync(0xffffffffu, nact > 0)) {
+      const bool up = (v & 16) != 0, odd = (v & 8) != 0;
+      const double r0 = __shfl_xor_sync(0xffffffffu, up ? f0 : f2, 16);
+      const double r1 = __shfl_xor_sync(0xffffffffu, f1, 16);
+      const double a0 = (up ? f2 : f0) + r0, a1 = f1 + r1;
+      fs = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        f0 += __shfl_xor_sync(0xffffffffu, f0, o);
-        f1 += __shfl_xor_sync(0xffffffffu, f1, o);
-        f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-      }
+      for (int o = 4; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      nact += __shfl_xor_sync(0xffffffffu, nact, o);
-      nadh += __shfl_xor_sync(0xffffffffu, nadh, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      const int g = v >> 5;
-      tf[0][g] = f0;
-      tf[1][g] = f1;
-      tf[2][g] = f2;
+    nact = (int)__reduce_add_sync(0xffffffffu, (unsigned)nact);
+    nadh = (int)__reduce_add_sync(0xffffffffu, (unsigned)nadh);
+    const int g = v >> 5, l = (int)threadIdx.x & 31;
+    if ((l & 7) == 0 && l < 24) tf[l >> 3][g] = fs;
+    if (l == 0) {
       ti[0][g] = nact;
       ti[1][g] = nadh;
     }
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  double F[3] = {0.0, 0.0, 0.0};
+  if (threadIdx.x >= 32) return;
+  double Fi = 0.0;
   int na = 0, nd = 0;
+#pragma unroll
   for (int k = 0; k < kTailLanes / 32; ++k) {
-    if (ti[0][k] > 0) {
-      F[0] += tf[0][k];
-      F[1] += tf[1][k];
-      F[2] += tf[2][k];
-    }
+    if (ti[0][k] > 0) Fi += tf[comp][k];
     na += ti[0][k];
     nd += ti[1][k];
   }
@@ -656,14 +685,28 @@ __device__ void tail_block(const Dev<T> &D, int mode) {
       c.mode = MODE_REPEAT;
     }
   } else {
-    // commit step n+1
-    for (int i = 0; i < 3; ++i) {
-      S.c[i] = ss.c[i];
-      S.w[i] = ss.w[i];
-      S.F[i] = F[i];
+    // commit step n+1, and the striker of the next step (Algorithm 1: the
+    // rigid instance moves first, with the contact force just committed)
+    const double ga = s_g - Fi * s_iM;
+    const double an = striker_along(__shfl_sync(0xffffffffu, ga, 0), __shfl_sync(0xffffffffu, ga, 1),
+                                    __shfl_sync(0xffffffffu, ga, 2), axis);
+    const double aI = an * (comp == 0 ? axis[0] : comp == 1 ? axis[1] : axis[2]);
+    double c1, w1;
+    striker_rk4(n_c, n_w, aI, D.dt, c1, w1);
+    if (lane0 < 3) {
+      D.imp->c[comp] = n_c;
+      D.imp->w[comp] = n_w;
+      D.imp->F[comp] = Fi;
+      D.imp_step->c[comp] = c1;
+      D.imp_step->w[comp] = w1;
+      D.imp_step->aI[comp] = aI;
     }
-    const double fc = F[0] * S.axis[0] + F[1] * S.axis[1] + F[2] * S.axis[2];
-    if (c.hist_count < D.hist_cap) D.fhist[c.hist_count++] = fc;
+    const double fc = striker_along(__shfl_sync(0xffffffffu, Fi, 0), __shfl_sync(0xffffffffu, Fi, 1),
+                                    __shfl_sync(0xffffffffu, Fi, 2), axis);
+    if (c.hist_count < D.hist_cap) {
+      if (lane0 == 0) D.fhist[c.hist_count] = fc;
+      ++c.hist_count;
+    }
     if (fc > c.f_peak) c.f_peak = fc;
     c.n_active = na;
     c.step += 1;
@@ -672,14 +715,8 @@ __device__ void tail_block(const Dev<T> &D, int mode) {
     c.hpar ^= 1;
     c.repeats = 0;
     c.mode = (c.step >= c.target) ? MODE_DONE : MODE_ADVANCE;
-    // striker of the next step (Algorithm 1: the rigid instance moves first,
-    // with the contact force just committed)
-    StrikerStep nx;
-    striker_rk4(S, D.dt, nx.c, nx.w, nx.aI);
-    *D.imp = S;
-    *D.imp_step = nx;
   }
-  *ctl = c;
+  if (lane0 == 0) *ctl = c;
 }
 
 // ---------------------------------------------------------------------------

@@ -40,11 +40,13 @@ __device__ __forceinline__ void pdl_enter() {
 // Kernels of a pass (one launch per step part); the per-item bodies are in
 // pdn_items.cuh, shared with the batched persistent kernel.
 template <typename T>
-__global__ void __launch_bounds__(kActRun) k_contact(Dev<T> D) {
+__global__ void __launch_bounds__(kActRun) k_contact(const __grid_constant__ Dev<T> D) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const ContactNode<T> q = contact_node(D, s);
   pdl_enter();
   const int mode = D.ctl->mode;
   if (mode != MODE_ADVANCE && mode != MODE_REPEAT) return;
-  const bool on = contact_item(D, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, mode);
+  const bool on = contact_item(D, s, mode, q);
   // the run's count of active nodes, for the tail's ordered list
   const int c = __syncthreads_count(on);
   if (D.act_cnt != nullptr && threadIdx.x == 0) D.act_cnt[blockIdx.x] = c;
@@ -342,12 +344,15 @@ __global__ void __launch_bounds__(256) k_gather_list(Dev<T> D, const int32_t *li
 
 // After pdn_set_impactor: the striker of the first step to be computed.
 __global__ void k_striker_init(Striker *S, StrikerStep *ss, double dt) {
-  double c1[3], w1[3], aI[3];
-  striker_rk4(*S, dt, c1, w1, aI);
+  double ga[3], axis[3];
   for (int i = 0; i < 3; ++i) {
-    ss->c[i] = c1[i];
-    ss->w[i] = w1[i];
-    ss->aI[i] = aI[i];
+    ga[i] = S->g[i] - S->F[i] * S->iM;
+    axis[i] = S->axis[i];
+  }
+  const double an = striker_along(ga[0], ga[1], ga[2], axis);
+  for (int i = 0; i < 3; ++i) {
+    ss->aI[i] = an * axis[i];
+    striker_rk4(S->c[i], S->w[i], ss->aI[i], dt, ss->c[i], ss->w[i]);
   }
 }
 

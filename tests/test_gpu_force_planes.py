@@ -91,6 +91,8 @@ def test_planes_equal_slots_in_a_batch(pkg, monkeypatch):
         for w, ctx in zip(ws, b.plates):
             Lx, Ly, H = w.plate.dims
             pkg.pdn_set_impactor(ctx, 4.0, 1e-5, (0.5 * Lx, 0.5 * Ly, H + 4.001), (0.0, 0.0, -3000.0))
+            pkg.pdn_set_state(ctx, *pi.seeded_state(w.plate, 7, amp=0.02, vamp=300.0,
+                                                    dimple=(0.5 * Lx, 0.5 * Ly, 0.12, 1.5)))
         pkg.pdn_batch_step(b, 100)
         out.append([pkg.pdn_get_state(ctx)[:2] for ctx in b.plates])
         b.close()
