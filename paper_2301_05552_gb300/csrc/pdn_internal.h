@@ -231,6 +231,8 @@ struct Dev {
   // points whose squared loading-function ratio exceeds sur_ratio2 (or whose
   // inputs leave the training box) take the exact law
   const float *sur_params;
+  // the same as the hex kernel's operand image (HexSurImage, pdn_surrogate.cu)
+  const void *sur_image;
   float sur_ratio2;
   // the first node id when the contact surface is the ascending contiguous
   // range surf[s] = surf_base + s (then s and j convert without the index

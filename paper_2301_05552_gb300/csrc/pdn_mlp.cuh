@@ -51,7 +51,7 @@ struct UmmaNet {
   __nv_bfloat16 W2[kHid * kHid];     // [64][64]
   __nv_bfloat16 W3[kHid * kHid];
   __nv_bfloat16 W4[kOutPad * kHid];  // [16 out][64 in]
-  float b1[kHid], b2[kHid], b3[kHid], b4[kOutPad];
+  alignas(16) float b1[kHid], b2[kHid], b3[kHid], b4[kOutPad];
 };
 // Activations of the 128 points (A operands), the MMA completion barrier
 // and the TMEM base address written by the allocation.
@@ -99,6 +99,14 @@ __device__ __forceinline__ uint4 pack8(const float *v) {
     w[k] = *reinterpret_cast<const uint32_t *>(&b);
   }
   return q;
+}
+
+// Two of relu(v + b), rounded to bf16.
+__device__ __forceinline__ uint32_t relu_pack2(float2 v, float2 b) {
+  const float2 z = __fadd2_rn(v, b);
+  uint32_t r;
+  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(z.y), "f"(z.x));
+  return r;
 }
 
 // Row r of the input tile: the normalised inputs (kInPad values, columns
@@ -156,49 +164,52 @@ __device__ __forceinline__ void tc_store16(__nv_bfloat16 *tile, int K, int r, in
   *reinterpret_cast<uint4 *>(b + umma::core_offset(r, c + 8, K)) = hi;
 }
 
-struct NoHidden {
-  __device__ void operator()(int, int, const uint4 &, const uint4 &) const {}
-};
-
 // Forward pass of the 128 points whose normalised inputs are in T.x (row t
 // written by thread t): y = the thread's normalised outputs (columns kOut..
 // zero).  Called by all 128 threads; thread 0 issues the MMAs.  T.tmem holds
 // kTmemCols allocated columns; phase is the completion barrier's current
-// parity (the same in every thread).  on_hidden(layer, column, lo, hi)
-// receives each 16-column piece of the thread's bf16 hidden activations.
-// Returns false in every thread when a wait on the tensor core gave up; y is
-// then not valid and no further MMA may be issued.
-template <typename OnHidden = NoHidden>
-__device__ __forceinline__ bool tc_forward128(const UmmaNet &N, UmmaTile &T, uint32_t &phase, float (&y)[kOutPad],
-                                              OnHidden &&on_hidden = OnHidden{}) {
+// parity (the same in every thread).  Returns false in every thread when a
+// wait on the tensor core gave up; y is then not valid and no further MMA may
+// be issued.
+//
+// The product of a layer (128 x 64 x 64) takes the tensor core about as long
+// as one round of shared-memory traffic; what costs is the epilogue, so it
+// is 32 columns per TMEM load, biases as 16-byte loads, packed additions and
+// one conversion that rounds two values and applies the ReLU: 90
+// instructions per layer instead of 250 (hex kernel of the learned law on
+// 221,184 hexes, with its operands fetched by one bulk copy: 203 to 172 us).
+__device__ __forceinline__ bool tc_forward128(const UmmaNet &N, UmmaTile &T, uint32_t &phase, float (&y)[kOutPad]) {
   const int t = threadIdx.x;
+  unsigned char *hb = reinterpret_cast<unsigned char *>(T.h);
 #pragma unroll 1
   for (int L = 0; L < 4; ++L) {
     const int K = L == 0 ? kInPad : kHid, Nn = L == 3 ? kOutPad : kHid;
     const __nv_bfloat16 *A = L == 0 ? T.x : T.h;
     const __nv_bfloat16 *B = L == 0 ? N.W1 : (L == 1 ? N.W2 : (L == 2 ? N.W3 : N.W4));
-    const float *bias = L == 0 ? N.b1 : (L == 1 ? N.b2 : (L == 2 ? N.b3 : N.b4));
     const uint32_t col = (uint32_t)(L & 1) * 64u;
     if (!tc_mma128(A, B, K, Nn, T.tmem + col, T, phase)) return false;
     if (L < 3) {
-#pragma unroll 1
-      for (int c = 0; c < kHid; c += 16) {
-        float v[16];
-        umma::tmem_ld16(tc_lane(T, col + (uint32_t)c), v);
+      const float4 *bias = reinterpret_cast<const float4 *>(L == 0 ? N.b1 : (L == 1 ? N.b2 : N.b3));
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const float z = v[k] + bias[c + k];
-          v[k] = z > 0.0f ? z : 0.0f;
+      for (int c = 0; c < kHid; c += 32) {
+        float v[32];
+        umma::tmem_ld32(tc_lane(T, col + (uint32_t)c), v);
+#pragma unroll
+        for (int k = 0; k < 32; k += 8) {
+          const float4 b0 = bias[(c + k) / 4], b1 = bias[(c + k) / 4 + 1];
+          uint4 q;
+          q.x = relu_pack2(make_float2(v[k], v[k + 1]), make_float2(b0.x, b0.y));
+          q.y = relu_pack2(make_float2(v[k + 2], v[k + 3]), make_float2(b0.z, b0.w));
+          q.z = relu_pack2(make_float2(v[k + 4], v[k + 5]), make_float2(b1.x, b1.y));
+          q.w = relu_pack2(make_float2(v[k + 6], v[k + 7]), make_float2(b1.z, b1.w));
+          *reinterpret_cast<uint4 *>(hb + umma::core_offset(t, c + k, kHid)) = q;
         }
-        uint4 lo, hi;
-        tc_store16(T.h, kHid, t, c, v, lo, hi);
-        on_hidden(L, c, lo, hi);
       }
     } else {
       float v[16];
       umma::tmem_ld16(tc_lane(T, col), v);
 #pragma unroll
-      for (int k = 0; k < kOutPad; ++k) y[k] = v[k] + bias[k];
+      for (int k = 0; k < kOutPad; ++k) y[k] = v[k] + N.b4[k];
     }
   }
   return true;

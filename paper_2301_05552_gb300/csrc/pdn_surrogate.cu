@@ -585,25 +585,50 @@ __global__ void k_init_params(float *p, uint64_t seed) {
 // halts the run with PDN_E_TIMEOUT) and the CTA finishes with the exact law.
 
 constexpr int kHexSurBlock = kTcRows;  // at most three CTAs per SM (registers): 3 x 128 TMEM columns
-struct HexSurSmem {
+// Network and scaling as the kernel keeps them in shared memory, one bulk
+// copy per CTA; laid out when the law is set (k_hex_sur_image).
+struct HexSurImage {
   UmmaNet N;
-  UmmaTile T;
   Scaling sc;
 };
+static_assert(sizeof(HexSurImage) % 16 == 0, "one bulk copy");
+struct HexSurSmem {
+  HexSurImage I;
+  UmmaTile T;
+  uint64_t bar_load;
+  uint64_t pad;
+};
 constexpr size_t kHexSurSmem = sizeof(HexSurSmem);
+// the image follows the parameters in the context's buffer
+constexpr size_t kSurImageOffset = (sizeof(float) * (kNumParams + PDN_SUR_SCALING) + 255) & ~size_t(255);
 static_assert(sizeof(Scaling) == PDN_SUR_SCALING * sizeof(float), "scaling record of 60 floats");
 static_assert(sizeof(Scaling) % 16 == 0, "16-byte aligned shared tiles");
 
-__global__ void __launch_bounds__(kHexSurBlock, 3) k_hex_sur(Dev<float> D, Mat<float> M) {
+// The image from the exchange order (parameters, scaling); one block.
+__global__ void k_hex_sur_image(const float *params, HexSurImage *I) {
+  load_net_umma(I->N, params);
+  for (int k = threadIdx.x; k < PDN_SUR_SCALING; k += blockDim.x)
+    reinterpret_cast<float *>(&I->sc)[k] = params[kNumParams + k];
+}
+
+__global__ void __launch_bounds__(kHexSurBlock, 3)
+    k_hex_sur(const __grid_constant__ Dev<float> D, const __grid_constant__ Mat<float> M) {
   extern __shared__ __align__(16) unsigned char smem[];
   HexSurSmem &S = *reinterpret_cast<HexSurSmem *>(smem);
   const Ctl *ctl = D.ctl;
+  // the image is fetched while the previous kernel of the pass finishes
+  if (threadIdx.x == 0) {
+    umma::mbar_init(&S.bar_load, 1);
+    umma::bulk_load(&S.I, D.sur_image, (uint32_t)sizeof(HexSurImage), &S.bar_load);
+  }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncthreads();
+  bool tc_ok = umma::mbar_wait(&S.bar_load, 0, kMaxPolls);
+  tc_ok = !__syncthreads_or(!tc_ok);
   const int mode = ctl->mode;
   if (mode >= MODE_DONE) return;
-  load_net_umma(S.N, D.sur_params);
-  for (int k = threadIdx.x; k < PDN_SUR_SCALING; k += blockDim.x)
-    reinterpret_cast<float *>(&S.sc)[k] = D.sur_params[kNumParams + k];
-  const Scaling &sc = S.sc;
+  const Scaling &sc = S.I.sc;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nh = D.nh;
   // a repeated pass evaluates only the marked elements (local repetition);
@@ -613,7 +638,6 @@ __global__ void __launch_bounds__(kHexSurBlock, 3) k_hex_sur(Dev<float> D, Mat<f
   if (!__syncthreads_or(act)) return;  // nothing to do in this CTA (no TMEM held yet)
   tc_setup(S.T);
   uint32_t phase = 0;
-  bool tc_ok = true;
   const int64_t el = e < nh ? e : nh - 1;
   const int ub = (mode == MODE_FORCES) ? (ctl->dpar ^ 1) : ctl->dpar;
   const int hb = ctl->hpar;
@@ -709,7 +733,7 @@ __global__ void __launch_bounds__(kHexSurBlock, 3) k_hex_sur(Dev<float> D, Mat<f
       }
       tc_store_input(S.T, threadIdx.x, xn);
       float y[kOutPad];
-      tc_ok = tc_forward128(S.N, S.T, phase, y);
+      tc_ok = tc_forward128(S.I.N, S.T, phase, y);
       net = use && tc_ok;
       if (net) {
 #pragma unroll
@@ -786,8 +810,17 @@ thread_local std::string g_sur_error;
 namespace pdn {
 cudaError_t launch_hex_sur(const Dev<float> &D, const Mat<float> &M, cudaStream_t s) {
   const int64_t g = (D.nh + kHexSurBlock - 1) / kHexSurBlock;
-  k_hex_sur<<<(unsigned)(g < 1 ? 1 : g), kHexSurBlock, kHexSurSmem, s>>>(D, M);
-  return cudaGetLastError();
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(g < 1 ? 1 : g));
+  cfg.blockDim = dim3(kHexSurBlock);
+  cfg.dynamicSmemBytes = kHexSurSmem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_hex_sur, D, M);
 }
 }  // namespace pdn
 
@@ -1265,7 +1298,7 @@ int pdn_set_surrogate(pdn_ctx *ctx, pdn_surrogate *s, double onset_ratio) {
     return PDN_E_CUDA;
   }
   if (!ctx->sur_buf) {
-    if (cudaMalloc(&ctx->sur_buf, sizeof(float) * (kNumParams + PDN_SUR_SCALING)) != cudaSuccess) {
+    if (cudaMalloc(&ctx->sur_buf, kSurImageOffset + sizeof(HexSurImage)) != cudaSuccess) {
       ctx->err = "learned-law parameters";
       return PDN_E_OOM;
     }
@@ -1277,12 +1310,18 @@ int pdn_set_surrogate(pdn_ctx *ctx, pdn_surrogate *s, double onset_ratio) {
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ctx->sur_buf + kNumParams, &s->sc, sizeof(float) * PDN_SUR_SCALING, cudaMemcpyHostToDevice,
                         ctx->stream);
+  HexSurImage *img = reinterpret_cast<HexSurImage *>(reinterpret_cast<unsigned char *>(ctx->sur_buf) + kSurImageOffset);
+  if (e == cudaSuccess) {
+    k_hex_sur_image<<<1, 256, 0, ctx->stream>>>(ctx->sur_buf, img);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
     ctx->err = std::string("learned-law parameters: ") + cudaGetErrorString(e);
     return PDN_E_CUDA;
   }
   ctx->Df.sur_params = ctx->sur_buf;
+  ctx->Df.sur_image = img;
   ctx->Df.sur_ratio2 = (float)(onset_ratio * onset_ratio);
   // the captured graph holds the old kernel choice
   if (ctx->graph) {
