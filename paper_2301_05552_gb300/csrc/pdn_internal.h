@@ -314,6 +314,10 @@ template <typename T>
 cudaError_t launch_pass(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_t gather_block,
                         cudaEvent_t *ev /* [6] or nullptr */, cudaStream_t side = nullptr,
                         cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
+// The element forces of D's committed state and their sum per node (Dev::fout)
+// alone: no contact, no tail (mode MODE_FORCES, no interfaces).
+template <typename T>
+cudaError_t launch_forces(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_t gather_block);
 cudaError_t launch_striker_init(Striker *S, StrikerStep *ss, double dt, cudaStream_t s);
 // Hex kernel with the learned law (pdn_surrogate.cu); D.sur_params != nullptr.
 cudaError_t launch_hex_sur(const Dev<float> &D, const Mat<float> &M, cudaStream_t s);

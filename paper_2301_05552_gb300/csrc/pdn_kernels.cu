@@ -637,6 +637,13 @@ cudaError_t launch_pass(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_
 }
 
 template <typename T>
+cudaError_t launch_forces(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_t gather_block) {
+  launch_hex(D, M, s);
+  launch_k(k_gather<T>, grid_of(D.nn, gather_block), gather_block, s, D);
+  return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_pairs_to_elements(const Dev<T> &D, cudaStream_t s) {
   if (D.ipair == nullptr || D.nc == 0) return cudaSuccess;
   k_pairs_to_elements<T><<<grid_of(D.nc, 256), 256, 0, s>>>(D);
@@ -670,6 +677,8 @@ template cudaError_t launch_pass<float>(const Dev<float> &, const Mat<float> &, 
                                         cudaEvent_t *, cudaStream_t, cudaEvent_t, cudaEvent_t);
 template cudaError_t launch_pass<double>(const Dev<double> &, const Mat<double> &, cudaStream_t, int32_t,
                                          cudaEvent_t *, cudaStream_t, cudaEvent_t, cudaEvent_t);
+template cudaError_t launch_forces<float>(const Dev<float> &, const Mat<float> &, cudaStream_t, int32_t);
+template cudaError_t launch_forces<double>(const Dev<double> &, const Mat<double> &, cudaStream_t, int32_t);
 template cudaError_t launch_box_records<float>(const Dev<float> &, float4 *, cudaStream_t);
 template cudaError_t launch_box_records<double>(const Dev<double> &, double4_32a *, cudaStream_t);
 template cudaError_t launch_pairs_to_elements<float>(const Dev<float> &, cudaStream_t);

@@ -67,8 +67,10 @@ struct PlyTable {
 // caller's csr_col: the element kernel writes each nodal force at its node's
 // CSR position), in one launch: each thread takes its node, its flag and its
 // slots.  One launch instead of two and a flag per element instead of 448
-// bytes of initial history: at 1,105 hexes in FP64 the call went from 143 us
-// to the figure in the notes below, of which the element kernel is most.
+// bytes of initial history, and neither the contact nor the tail kernel of a
+// pass: at 1,105 hexes in FP64 the call went from 143 us to 33 us with the
+// lanes-of-eight element kernel and to 28 us with three launches instead of
+// five, of which the element kernel is most.
 template <typename T>
 __global__ void k_noalloc_prepare(Ctl *ctl, const double *X, const double *d, typename Vec4T<T>::type *X4,
                                   typename Vec4T<T>::type *u4, int64_t nn, uint8_t *flag, int64_t nh,
@@ -76,6 +78,9 @@ __global__ void k_noalloc_prepare(Ctl *ctl, const double *X, const double *d, ty
                                   const __grid_constant__ PlyTable<T> tab) {
   using V4 = typename Vec4T<T>::type;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // the element kernel's blocks take their places meanwhile (they wait for
+  // this grid's end before they read anything)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (i == 0) {
     Ctl c{};
     c.mode = MODE_FORCES;
@@ -150,7 +155,7 @@ cudaError_t run_noalloc(unsigned char *base, int64_t nn, int64_t nh, const int32
                                                n_plies, tab);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_pass<T>(D, M, s, kBlock, nullptr);
+  return launch_forces<T>(D, M, s, kBlock);
 }
 
 }  // namespace
