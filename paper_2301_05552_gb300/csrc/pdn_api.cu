@@ -1286,7 +1286,6 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     }
     D.fe = planes ? nullptr : reinterpret_cast<V4 *>(d_fe);
     D.fplane = planes ? reinterpret_cast<float *>(d_fe) : nullptr;
-    D.fplane_n = plane_n;
     D.rel = d_rel;
     D.act_cnt = P.act_cnt;
     // PDN_FULL_REPEAT=1: repeated passes evaluate every element and node
@@ -1303,6 +1302,17 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     D.coh_w = (T)coh_w;
     for (int b = 0; b < 2; ++b) D.rDn[b] = pairs_on ? reinterpret_cast<T *>(P.rDn[b]) : nullptr;
     D.pair_layer = pair_layer;
+    // with s = ceil(log2 L) and m = floor(2^(31 + s) / L) + 1 the error of
+    // j m / 2^(31 + s) stays below 1 / L for j < 2^31 (m < 2^32; L >= 2: a
+    // quadrilateral's nodes share a layer)
+    D.pair_mul = 0;
+    D.pair_shift = 0;
+    if (pair_layer > 1) {
+      int s2 = 1;
+      while ((int64_t(1) << s2) < pair_layer) ++s2;
+      D.pair_mul = (uint32_t)(((uint64_t(1) << (31 + s2)) / (uint64_t)pair_layer) + 1);
+      D.pair_shift = s2 - 1;
+    }
     D.slot_compact = slot_compact ? 1 : 0;
     D.pair_inv_L = pair_layer > 0 ? 1.0f / (float)pair_layer : 0.0f;
     for (int l = 0; l < kMaxPairLayers; ++l) D.layer_off[l] = layer_off[l];

@@ -54,32 +54,50 @@ __device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a
 // 30x slower than the integer pipe, and the node update needs six per node.
 // Zeros and normal numbers take the integer path; subnormals, infinities,
 // NaNs and out-of-range values fall back to the hardware conversion.
-__device__ __forceinline__ double to_f64(float f) {
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t ex = (u >> 23) & 0xffu;
-  const uint32_t sign = u & 0x80000000u;
-  if ((u & 0x7fffffffu) == 0u) return __hiloint2double((int)sign, 0);
-  if (ex == 0u || ex == 0xffu) return (double)f;
-  const uint32_t man = u & 0x7fffffu;
-  const uint32_t hi = sign | ((ex + (1023u - 127u)) << 20) | (man >> 3);
-  return __hiloint2double((int)hi, (int)(man << 29));
+// Three at once: one test for all, so a node takes one branch.
+__device__ __forceinline__ void to_f64(const float (&f)[3], double (&d)[3]) {
+  bool rare = false;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t u = __float_as_uint(f[i]), t = u & 0x7fffffffu;
+    const uint32_t hi = (t == 0u ? 0u : (t >> 3) + (896u << 20)) | (u & 0x80000000u);
+    d[i] = __hiloint2double((int)hi, (int)(u << 29));
+    rare = rare || (t - 0x00800000u >= 0x7f000000u && t != 0u);
+  }
+  if (rare) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) d[i] = (double)f[i];
+  }
 }
-__device__ __forceinline__ double to_f64(double d) { return d; }
+__device__ __forceinline__ void to_f64(const double (&f)[3], double (&d)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) d[i] = f[i];
+}
 
-// Round to nearest, ties to even.
-__device__ __forceinline__ float to_elem(double d, float) {
-  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
-  const uint32_t ex = (hi >> 20) & 0x7ffu;
-  const uint32_t sign = hi & 0x80000000u;
-  if ((hi & 0x7fffffffu) == 0u && lo == 0u) return __uint_as_float(sign);
-  if (ex < 897u || ex > 1150u) return (float)d;  // float subnormal / overflow range or inf/nan
-  const uint32_t m = ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const uint32_t rest = lo & 0x1fffffffu;
-  uint32_t bits = sign | ((ex - 896u) << 23) | m;
-  if (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) bits += 1u;
-  return __uint_as_float(bits);
+// Round to nearest, ties to even: the exponent's low bits and the 23 leading
+// mantissa bits by one funnel shift, the bias by a wrapping addition.
+__device__ __forceinline__ void to_elem(const double (&d)[3], float (&f)[3]) {
+  bool rare = false;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const uint32_t hi = (uint32_t)__double2hiint(d[i]), lo = (uint32_t)__double2loint(d[i]);
+    const uint32_t t = hi & 0x7fffffffu;
+    const bool zero = (t | lo) == 0u;
+    uint32_t bits = __funnelshift_l(lo, hi, 3) + 0x40000000u;
+    bits += ((lo & 0x1fffffffu) + (bits & 1u)) > 0x10000000u ? 1u : 0u;
+    f[i] = __uint_as_float((zero ? 0u : bits & 0x7fffffffu) | (hi & 0x80000000u));
+    // outside float's normal range (897 <= exponent <= 1150): subnormal, overflow, inf, nan
+    rare = rare || (t - (897u << 20) >= (254u << 20) && !zero);
+  }
+  if (rare) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[i] = (float)d[i];
+  }
 }
-__device__ __forceinline__ double to_elem(double d, double) { return d; }
+__device__ __forceinline__ void to_elem(const double (&d)[3], double (&f)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) f[i] = d[i];
+}
 
 // Natural-coordinate signs of hex8 node a (bottom face CCW, then top face).
 __host__ __device__ constexpr int sgn_x(int a) { return ((a ^ (a >> 1)) & 1) ? 1 : -1; }
@@ -274,15 +292,20 @@ __device__ __forceinline__ void element_slots(const Dev<T> &D, const int32_t *co
 // Force planes (Dev::fplane).  A slot of 16 bytes per node and rank makes
 // every store of a warp (one corner of 32 consecutive elements) and every load
 // of the gather touch 32 cache lines, 12 bytes of each; where consecutive
-// elements have consecutive nodes, planes turn both into full 128-byte lines
-// and drop the fourth component.  GB300, with the slots' time
+// elements have consecutive nodes, planes turn both into whole 128-byte lines
+// and drop the fourth component.  The planes of 32 nodes lie together (3 KB),
+// so that a gather warp reads one piece of memory and addresses it with
+// constant offsets.  GB300, with the slots' time
 // first: 7.68 M hexes 1.065 -> 0.943 ms per step, 393,216 hexes 90 -> 85 us,
 // 228,528 70 -> 66 us, 69,540 general hexes 41 -> 39 us.
-__device__ __forceinline__ void plane_store(float *plane, int64_t n, int r, int nd, float fx, float fy, float fz) {
-  float *p = plane + (int64_t)(3 * r) * n + nd;
+__device__ __forceinline__ float *plane_of(float *planes, uint32_t j) {
+  return planes + ((size_t)(j >> 5) * (24 * 32) + (j & 31u));
+}
+__device__ __forceinline__ void plane_store(float *planes, int r, int nd, float fx, float fy, float fz) {
+  float *p = plane_of(planes, (uint32_t)nd) + 96 * r;
   p[0] = fx;
-  p[n] = fy;
-  p[2 * n] = fz;
+  p[32] = fy;
+  p[64] = fz;
 }
 // The eight nodal forces f (by corner) of element e (hexes, then interfaces;
 // conn: its kind's connectivity, el: its index there) into the planes.
@@ -294,20 +317,19 @@ __device__ __forceinline__ void plane_store8(const Dev<float> &D, const int32_t 
   const uint32_t rk = __ldg(D.rank + e);
 #pragma unroll
   for (int a = 0; a < 8; ++a)
-    plane_store(D.fplane, D.fplane_n, (int)((rk >> (3 * a)) & 7u), nd[a], f[a][0], f[a][1], f[a][2]);
+    plane_store(D.fplane, (int)((rk >> (3 * a)) & 7u), nd[a], f[a][0], f[a][1], f[a][2]);
 }
 // Slots K0 .. K1 - 1 of node j: from its planes, or from its slots fs.
 template <int K0, int K1, typename T, typename V4>
 __device__ __forceinline__ void load_slots(const Dev<T> &D, const V4 *fs, int64_t j, V4 (&f)[8]) {
   if constexpr (sizeof(T) == 4) {
     if (D.fplane != nullptr) {
-      const float *p = D.fplane + j;
-      const int64_t n = D.fplane_n;
+      const float *p = plane_of(D.fplane, (uint32_t)j);
 #pragma unroll
       for (int k = K0; k < K1; ++k) {
-        f[k].x = p[(3 * k) * n];
-        f[k].y = p[(3 * k + 1) * n];
-        f[k].z = p[(3 * k + 2) * n];
+        f[k].x = p[96 * k];
+        f[k].y = p[96 * k + 32];
+        f[k].z = p[96 * k + 64];
       }
       return;
     }

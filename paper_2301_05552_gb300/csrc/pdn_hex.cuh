@@ -303,7 +303,7 @@ __device__ __forceinline__ void hex_lanes8_item(const Dev<T> &D, const Mat<T> &M
   if (mode == MODE_REPEAT && D.rmark_n != nullptr) D.rmark_n[r.nd] = 1;
   if constexpr (sizeof(T) == 4) {
     if (D.fplane != nullptr) {
-      plane_store(D.fplane, D.fplane_n, (int)((__ldg(D.rank + e) >> (3 * r.a)) & 7u), r.nd, r.f[0], r.f[1], r.f[2]);
+      plane_store(D.fplane, (int)((__ldg(D.rank + e) >> (3 * r.a)) & 7u), r.nd, r.f[0], r.f[1], r.f[2]);
       return;
     }
   }

@@ -179,11 +179,10 @@ struct Dev {
   uint8_t *pflag[2];       // [nh]
   uint8_t *cflag[2];       // [nc]
   V4 *fe;                  // [(nh + nc) * 8] element nodal forces
-  // FP32 element forces as planes: component i of the slot of rank r of node j
-  // at fplane[(3 r + i) fplane_n + j] (fplane_n: nn rounded up to 32); fe is
+  // FP32 element forces as planes of 32 nodes: component i of the slot of rank
+  // r of node j at fplane[24 * 32 * (j / 32) + 32 (3 r + i) + j % 32]; fe is
   // then not used.  Null: slots of fe.
   float *fplane;
-  int64_t fplane_n;
   // contact
   uint8_t *act[2];         // [ns] contact set by step parity
   uint8_t *rel;            // [ns] released in the current step
@@ -270,6 +269,9 @@ struct Dev {
   // upper side of an interface; node flag bits 4-6 hold the count of a node's
   // interface elements.  0: partners from ipair (a second load round).
   int32_t pair_layer;
+  // j / pair_layer = umulhi(j, pair_mul) >> pair_shift for every j < 2^31
+  uint32_t pair_mul;
+  int32_t pair_shift;
   uint64_t pair_mask[2][2];
   // compact force slots of a layered numbering with node pairs: a node of an
   // interface layer owns 4 slots (it has at most four hexes and its
