@@ -490,13 +490,13 @@ void launch_elem(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
 // FP64 boxes: one thread per element or eight lanes.  An FP64 operation holds
 // its scheduler 64 cycles whether one warp or more are resident, so the
 // launch takes (warps on the fullest scheduler) x (operations per warp): about
-// 900 per warp of 32 elements, or 190 per warp of 4.
+// 900 per warp of 32 elements, or 170 per warp of 4.
 template <typename T>
 bool hex_lanes8_fits(const Dev<T> &D) {
   if (sizeof(T) == 4) return false;
   const int64_t schedulers = 4 * 152;
   const int64_t w1 = (D.nh + 31) / 32, w8 = (D.nh + 3) / 4;
-  return (w8 + schedulers - 1) / schedulers * 190 <= (w1 + schedulers - 1) / schedulers * 900;
+  return (w8 + schedulers - 1) / schedulers * 170 <= (w1 + schedulers - 1) / schedulers * 900;
 }
 
 template <typename T>
