@@ -101,12 +101,23 @@ __device__ __forceinline__ uint4 pack8(const float *v) {
   return q;
 }
 
-// Two of relu(v + b), rounded to bf16.
+// Two of relu(v + b), rounded to bf16 (rounding keeps order and sign, so the
+// maximum is taken on the rounded pair; a NaN becomes 0, as in z > 0 ? z : 0).
 __device__ __forceinline__ uint32_t relu_pack2(float2 v, float2 b) {
   const float2 z = __fadd2_rn(v, b);
-  uint32_t r;
-  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(z.y), "f"(z.x));
-  return r;
+  const __nv_bfloat162 r = __hmax2(__floats2bfloat162_rn(z.x, z.y), __float2bfloat162_rn(0.0f));
+  return *reinterpret_cast<const uint32_t *>(&r);
+}
+
+// Eight of them as one 16-byte core-matrix row.
+__device__ __forceinline__ uint4 relu_pack8(const float *v, const float4 *bias) {
+  const float4 b0 = bias[0], b1 = bias[1];
+  uint4 q;
+  q.x = relu_pack2(make_float2(v[0], v[1]), make_float2(b0.x, b0.y));
+  q.y = relu_pack2(make_float2(v[2], v[3]), make_float2(b0.z, b0.w));
+  q.z = relu_pack2(make_float2(v[4], v[5]), make_float2(b1.x, b1.y));
+  q.w = relu_pack2(make_float2(v[6], v[7]), make_float2(b1.z, b1.w));
+  return q;
 }
 
 // Row r of the input tile: the normalised inputs (kInPad values, columns
@@ -175,9 +186,10 @@ __device__ __forceinline__ void tc_store16(__nv_bfloat16 *tile, int K, int r, in
 // The product of a layer (128 x 64 x 64) takes the tensor core about as long
 // as one round of shared-memory traffic; what costs is the epilogue, so it
 // is 32 columns per TMEM load, biases as 16-byte loads, packed additions and
-// one conversion that rounds two values and applies the ReLU: 90
-// instructions per layer instead of 250 (hex kernel of the learned law on
-// 221,184 hexes, with its operands fetched by one bulk copy: 203 to 172 us).
+// the ReLU on packed pairs: 120 instructions per layer instead of 250 (learned
+// law on 221,184 hexes, with its operands fetched by one bulk copy: step 254 to
+// 222 us at three CTAs per SM; the ReLU by cvt.rn.relu would be 4 % faster but
+// keeps a NaN).
 __device__ __forceinline__ bool tc_forward128(const UmmaNet &N, UmmaTile &T, uint32_t &phase, float (&y)[kOutPad]) {
   const int t = threadIdx.x;
   unsigned char *hb = reinterpret_cast<unsigned char *>(T.h);
@@ -196,13 +208,7 @@ __device__ __forceinline__ bool tc_forward128(const UmmaNet &N, UmmaTile &T, uin
         umma::tmem_ld32(tc_lane(T, col + (uint32_t)c), v);
 #pragma unroll
         for (int k = 0; k < 32; k += 8) {
-          const float4 b0 = bias[(c + k) / 4], b1 = bias[(c + k) / 4 + 1];
-          uint4 q;
-          q.x = relu_pack2(make_float2(v[k], v[k + 1]), make_float2(b0.x, b0.y));
-          q.y = relu_pack2(make_float2(v[k + 2], v[k + 3]), make_float2(b0.z, b0.w));
-          q.z = relu_pack2(make_float2(v[k + 4], v[k + 5]), make_float2(b1.x, b1.y));
-          q.w = relu_pack2(make_float2(v[k + 6], v[k + 7]), make_float2(b1.z, b1.w));
-          *reinterpret_cast<uint4 *>(hb + umma::core_offset(t, c + k, kHid)) = q;
+          *reinterpret_cast<uint4 *>(hb + umma::core_offset(t, c + k, kHid)) = relu_pack8(v + k, bias + (c + k) / 4);
         }
       }
     } else {

@@ -132,8 +132,11 @@ __global__ void k_law_points(LawArgs A, const float *in, float *out, int64_t n) 
 //    previous update runs.
 // Sums keep one order (points within a tile, tiles in order), so a run gives
 // the same parameters whatever the launch.  GB300, 8,192 points (64 CTAs):
-// 16.8 us per iteration, against 97 us for separate tile, weight-gradient
-// and update kernels that passed everything through memory.
+// 15.1 us per iteration, against 97 us for separate tile, weight-gradient
+// and update kernels that passed everything through memory.  Of a tile's 17,800
+// cycles after the wait the epilogues and the write of dW were most (a wait on
+// the tensor core is 230 to 600): packed epilogues with static addresses and dW
+// written in lines took it from 16.8 us.
 
 // The weights as BF16 operands: forward (UmmaNet, with the FP32 biases) and
 // transposed (row n: the weights from input n to every output) for the
@@ -207,7 +210,7 @@ __device__ __forceinline__ void issue_wgrad(const __nv_bfloat16 *G, int ng, cons
 // its point) from the rows of X (raw inputs) and Tgt (raw targets), drawn by a
 // seeded hash when random, scaled by sc.  Loss = mean over points and the kOut
 // outputs of (y_n - t_n)^2; its partial is per CTA (loss_part), and so are the
-// weight and bias gradients (partW [layer][tile][out][in], partB
+// weight and bias gradients (partW [layer][tile][in][64 out], partB
 // [layer][tile][out]).  A wait that gives up sets *status to PDN_E_TIMEOUT.
 __global__ void __launch_bounds__(kTrainThreads, 1)
     k_train_tile(const TrainImage *img, const __grid_constant__ Scaling sc, const float *X, const float *Tgt,
@@ -246,8 +249,9 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   const uint32_t lane_base = S.tmem + ((uint32_t)(warp & 3) << 21);
   uint32_t phase = 0;
   float y[kOutPad];
-#pragma unroll 1
-  for (int L = 0; L < 4 && ok; ++L) {
+#pragma unroll
+  for (int L = 0; L < 4; ++L) {
+    if (!ok) break;
     const uint32_t col = (uint32_t)(L & 1) * 64u;
     if (L > 0) {
       umma::fence_before_sync();
@@ -264,22 +268,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     ok = train_wait(&S.bar, phase);
     phase ^= 1u;
     if (!ok) break;
-    const float *bias = L == 0 ? S.W.N.b1 : (L == 1 ? S.W.N.b2 : (L == 2 ? S.W.N.b3 : S.W.N.b4));
     if (L < 3) {
+      const float4 *bias = reinterpret_cast<const float4 *>((L == 0 ? S.W.N.b1 : (L == 1 ? S.W.N.b2 : S.W.N.b3)) + c0);
+      unsigned char *hb = reinterpret_cast<unsigned char *>(S.h[L < 3 ? L : 0]) + umma::core_offset(r, c0, kHid);
       float v[32];
       umma::tmem_ld32(lane_base + col + (uint32_t)c0, v);
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const float z = v[k] + bias[c0 + k];
-        v[k] = z > 0.0f ? z : 0.0f;
-      }
-      unsigned char *hb = reinterpret_cast<unsigned char *>(S.h[L]);
-#pragma unroll
-      for (int k = 0; k < 32; k += 8) *reinterpret_cast<uint4 *>(hb + umma::core_offset(r, c0 + k, kHid)) = pack8(v + k);
+      for (int k = 0; k < 32; k += 8) *reinterpret_cast<uint4 *>(hb + 16 * k) = relu_pack8(v + k, bias + k / 4);
     } else if (t < kTcRows) {
       umma::tmem_ld16(lane_base + col, y);
 #pragma unroll
-      for (int k = 0; k < kOutPad; ++k) y[k] += bias[k];
+      for (int k = 0; k < kOutPad; ++k) y[k] += S.W.N.b4[k];
     }
   }
   float lsum = 0.0f;
@@ -319,8 +318,9 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   };
   // back through the hidden layers: dZ_L = (dZ_{L+1} W_{L+1}) * relu'(h_L);
   // the weight gradient of layer L + 1 follows its dZ into the queue
-#pragma unroll 1
-  for (int L = 2; L >= 0 && ok; --L) {
+#pragma unroll
+  for (int L = 2; L >= 0; --L) {
+    if (!ok) break;
     const uint32_t col = (uint32_t)(L & 1) * 64u;
     umma::fence_before_sync();
     umma::fence_smem_to_async();
@@ -375,16 +375,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   }
   if (ok && (warp & 3) < 2) {
     // rows (outputs) 0..63 of dW are lanes 0..63: warps 0 and 1 write layers 2
-    // and 1, warps 4 and 5 layers 3 and 4
+    // and 1, warps 4 and 5 layers 3 and 4, input by input, so that a warp's
+    // store is one line (row by row it is 32 sectors: 1.7 us of the kernel)
     auto write = [&](int layer, uint32_t col, int K) {
-      float *pW = partW + ((size_t)layer * n_tiles + tile) * (kHid * kHid) + r * K;
+      float *pW = partW + ((size_t)layer * n_tiles + tile) * (kHid * kHid) + r;
+#pragma unroll
       for (int c = 0; c < K; c += 16) {
         float v[16];
         umma::tmem_ld16(lane_base + col + (uint32_t)c, v);
         if (r < layer_out(layer)) {
 #pragma unroll
-          for (int k = 0; k < 16; k += 4)
-            *reinterpret_cast<float4 *>(pW + c + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+          for (int k = 0; k < 16; ++k) pW[(c + k) * kHid] = v[k];
         }
       }
     };
@@ -469,14 +470,26 @@ __global__ void __launch_bounds__(128) k_train_update(float *params, float *m1, 
                                                       TrainImage *img, const float *partW, const float *partB,
                                                       int64_t n_tiles, float lr, float bc1, float bc2) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  int layer = 0, row = 0, col = 0;
-  if (p < kNumParams) param_site(p, layer, row, col);
+  // consecutive threads take consecutive outputs of one input, as the partials
+  // lie: a matrix is numbered column by column, p its place in the exchange order
+  const int q0 = blockIdx.x * blockDim.x + threadIdx.x;
+  int p = q0, layer = 0, row = 0, col = 0;
+  if (q0 < kNumParams) {
+    param_site(q0, layer, row, col);
+    if (col >= 0) {
+      const int in = layer == 0 ? kIn : kHid, out = layer == 3 ? kOut : kHid;
+      const int k = row * in + col;
+      p = q0 - k;
+      row = k % out;
+      col = k / out;
+      p += row * in + col;
+    }
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (p >= kNumParams) return;
+  if (q0 >= kNumParams) return;
   const int64_t stride = col < 0 ? kHid : kHid * kHid;
   const float *src = col < 0 ? partB + (int64_t)layer * n_tiles * kHid + row
-                             : partW + (int64_t)layer * n_tiles * (kHid * kHid) + row * layer_in(layer) + col;
+                             : partW + (int64_t)layer * n_tiles * (kHid * kHid) + col * kHid + row;
   float m0 = 0.0f, v0 = 0.0f, w0 = 0.0f;
   if (lr > 0.0f) {
     m0 = m1[p];
@@ -587,7 +600,8 @@ __global__ void k_init_params(float *p, uint64_t seed) {
 // Four CTAs per SM (128 registers, 62 bytes of spills): 4 x 128 TMEM columns, all
 // there are.  With three (168 registers) 36 % of the issue slots were used, the
 // rest waiting for the tensor core and TMEM, and 1,728 CTAs took 3.8 waves
-// instead of 2.8: step of 221,184 hexes 222 against 198 us.
+// instead of 2.8: step of 221,184 hexes 222 against 198 us (206 us with the
+// ReLU that turns a NaN into 0, in pdn_mlp.cuh).
 constexpr int kHexSurBlock = kTcRows;
 // Network and scaling as the kernel keeps them in shared memory, one bulk
 // copy per CTA; laid out when the law is set (k_hex_sur_image).
