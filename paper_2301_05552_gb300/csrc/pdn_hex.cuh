@@ -695,7 +695,7 @@ __device__ __noinline__ void hex_box_slow(const Dev<T> *D, const Mat<T> *M, int6
 // element (valid = false: none).  Returns valid (false too where a repeated
 // pass does not evaluate the element).
 template <typename T>
-__device__ __forceinline__ bool hex_box_forces(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode,
+__device__ __forceinline__ bool hex_box_pairs_core(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode,
                                                T (&f)[8][3], int (&nd)[8]) {
   using V4 = typename Vec4T<T>::type;
   constexpr uint32_t kAll = 0xffffffffu;
@@ -761,33 +761,6 @@ __device__ __forceinline__ bool hex_box_forces(const Dev<T> &D, const Mat<T> &M,
     }
   }
   return valid;
-}
-
-// One box per thread; the warp calls together.
-template <typename T>
-__device__ __forceinline__ void hex_box_item(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode) {
-  using V4 = typename Vec4T<T>::type;
-  T f[8][3];
-  int nd[8];
-  if (!hex_box_forces(D, M, e, valid, mode, f, nd)) return;
-  if constexpr (sizeof(T) == 4) {
-    if (D.fplane != nullptr) {
-      plane_store8(D, D.hex, e, e, f);
-      return;
-    }
-  }
-  const uint32_t rk = D.rank != nullptr ? __ldg(D.rank + e) : 0u;
-  int ps[8];
-  element_slots(D, D.hex, e, reinterpret_cast<const int4 *>(D.pos) + 2 * e, rk, ps);
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    V4 o;
-    o.x = f[a][0];
-    o.y = f[a][1];
-    o.z = f[a][2];
-    o.w = T(0);
-    D.fe[ps[a]] = o;
-  }
 }
 
 }  // namespace detail

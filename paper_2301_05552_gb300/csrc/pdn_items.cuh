@@ -186,13 +186,40 @@ __device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mod
 // ---------------------------------------------------------------------------
 // Kernel 2: hex8 internal forces of an item (pdn_hex.cuh): boxes one element
 // per thread (the warp calls together), other hexes eight lanes per element.
+// One box per thread; the warp calls together.
+template <typename T>
+__device__ __forceinline__ void hex_item_box_pairs(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode) {
+  using V4 = typename Vec4T<T>::type;
+  T f[8][3];
+  int nd[8];
+  if (!hex_box_pairs_core(D, M, e, valid, mode, f, nd)) return;
+  if constexpr (sizeof(T) == 4) {
+    if (D.fplane != nullptr) {
+      plane_store8(D, D.hex, e, e, f);
+      return;
+    }
+  }
+  const uint32_t rk = D.rank != nullptr ? __ldg(D.rank + e) : 0u;
+  int ps[8];
+  element_slots(D, D.hex, e, reinterpret_cast<const int4 *>(D.pos) + 2 * e, rk, ps);
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    V4 o;
+    o.x = f[a][0];
+    o.y = f[a][1];
+    o.z = f[a][2];
+    o.w = T(0);
+    D.fe[ps[a]] = o;
+  }
+}
+
 template <typename T, bool BOX>
 __device__ __forceinline__ void hex_item(const Dev<T> &D, const Mat<T> &M, int64_t first, int64_t end, int mode) {
   // elements [first, end) of this block, strided over its threads
   const int lane = (int)(threadIdx.x & 31);
   if constexpr (BOX) {
     for (int64_t i = first + (int)(threadIdx.x & ~31u); i < end; i += blockDim.x)
-      hex_box_item(D, M, i + lane, i + lane < end, mode);
+      hex_item_box_pairs(D, M, i + lane, i + lane < end, mode);
   } else {
     for (int64_t i = 8 * first + (int)(threadIdx.x & ~31u); i < 8 * end; i += blockDim.x)
       hex_lanes8_item<T, false>(D, M, i + lane, end, mode);

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(128, MINB) k_hex(const __grid_constant__ Dev<T
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  hex_box_item(D, M, e, e < D.nh, mode);
+  hex_item_box_pairs(D, M, e, e < D.nh, mode);
 }
 
 // Eight lanes per element: general hexes, and boxes in launches too small to
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
       if (S.kind[k] == 0) {
         float f[8][3];
         int nd[8];
-        if (hex_box_forces(D, M, el, col, mode, f, nd)) store(f, nd);
+        if (hex_box_pairs_core(D, M, el, col, mode, f, nd)) store(f, nd);
       } else if (col) {
         coh_forces<float, true>(D, M, el, mode, store);
       }
