@@ -117,16 +117,21 @@ __device__ __forceinline__ LaneForce<T> hex_lanes8(const Dev<T> &D, const Mat<T>
     g[2] = interp(interp(diff(v, 2), 0), 1);
   };
   T H[3][3], Ji[3][3], det = T(0), wk[3], vol;
-  if constexpr (BOX) {
-    // the box record's reciprocals and volume instead of differences and a
-    // reciprocal of the coordinates; the scale of direction k goes into its
-    // last interpolation (FP64: 170 operations of this element, 193 before)
+  // FP64 boxes take the box record's reciprocals and volume, with the scale of
+  // direction k in its last interpolation: 170 FP64 operations instead of the
+  // 193 with differences and a reciprocal of the coordinates (8,192 hexes on
+  // GB300: 48.6 to 45.3 us per step).  In FP32 the operations are not what
+  // bounds the element, and the coordinates' differences round once less.
+  constexpr bool REC = BOX && sizeof(T) == 8;
+  auto scaled = [&](T v, int m, T s) {
+    return rfma(rmul(al, s), v, rmul(rmul(be, s), __shfl_xor_sync(kAll, v, 1 << m)));
+  };
+  if constexpr (REC) {
     const V4 box = D.box[ee];
     const T jd[3] = {box.x, box.y, box.z};
     vol = rmul(T(8), box.w);
 #pragma unroll
     for (int k = 0; k < 3; ++k) wk[k] = rmul(box.w, jd[k]);
-    auto scaled = [&](T v, int m, T s) { return rfma(rmul(al, s), v, rmul(rmul(be, s), __shfl_xor_sync(kAll, v, 1 << m))); };
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const T vz = interp(un[i], 2);
@@ -134,6 +139,28 @@ __device__ __forceinline__ LaneForce<T> hex_lanes8(const Dev<T> &D, const Mat<T>
       H[i][1] = scaled(diff(vz, 1), 0, jd[1]);
       H[i][2] = scaled(interp(diff(un[i], 2), 0), 1, jd[2]);
     }
+  } else if constexpr (BOX) {
+    const V4 x = D.X4[nd];
+    const T xn[3] = {x.x, x.y, x.z};
+    T hx[3], jd[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) hx[k] = diff(xn[k], k);
+    // one reciprocal per lane, shared by the group
+    const int k3 = sub % 3;
+    const T r = xrcp(k3 == 0 ? hx[0] : k3 == 1 ? hx[1] : hx[2]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) jd[k] = __shfl_sync(kAll, r, (lane & 24) + k);
+    vol = rmul(hx[0], rmul(hx[1], hx[2]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      T g[3];
+      grad(un[i], g);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) H[i][k] = rmul(g[k], jd[k]);
+    }
+    wk[0] = rmul(T(0.125), rmul(hx[1], hx[2]));
+    wk[1] = rmul(T(0.125), rmul(hx[0], hx[2]));
+    wk[2] = rmul(T(0.125), rmul(hx[0], hx[1]));
   } else {
     const V4 x = D.X4[nd];
     const T xn[3] = {x.x, x.y, x.z};
@@ -247,7 +274,12 @@ __device__ __forceinline__ LaneForce<T> hex_lanes8(const Dev<T> &D, const Mat<T>
 #pragma unroll
     for (int i = 0; i < 3; ++i)
       Q[k][i] = rfma(S[k][2], H[i][2], rfma(S[k][1], H[i][1], rfma(S[k][0], H[i][0], S[k][i])));
-  if constexpr (!BOX) {
+  if constexpr (BOX && !REC) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Q[k][i] = rmul(wk[k], Q[k][i]);
+  } else if constexpr (!BOX) {
     // det J J^-1 P / 2 = cofactors P / 8
     T R[3][3];
 #pragma unroll
@@ -270,8 +302,7 @@ __device__ __forceinline__ LaneForce<T> hex_lanes8(const Dev<T> &D, const Mat<T>
       return bit[k] ? s : -s;
     };
     T t0, t1, t2;
-    if constexpr (BOX) {
-      auto scaled = [&](T v, int m, T s) { return rfma(rmul(al, s), v, rmul(rmul(be, s), __shfl_xor_sync(kAll, v, 1 << m))); };
+    if constexpr (REC) {
       t0 = scaled(pair(Q[0][i], 0), 1, wk[0]);
       t1 = scaled(pair(Q[1][i], 1), 0, wk[1]);
       t2 = scaled(interp(pair(Q[2][i], 2), 0), 1, wk[2]);
