@@ -1338,18 +1338,23 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
     D.ell = ell ? 1 : 0;
     D.surf_base = surf_base;
   };
+  // The ply table on the context's stream, where the first pass reads it: the
+  // uploads above were complete with cudaDeviceSynchronize, and a copy on the
+  // default stream is not ordered with a stream that does not block on it.
+  std::vector<double> ply_q64;  // until the stream has been waited for (prime_state)
+  std::vector<float> ply_q32;
+  auto up_table = [&](auto &q, const auto &D, auto *box) {
+    q.resize((size_t)kPlyStride<std::decay_t<decltype(q[0])>> * mesh->n_plies);
+    ply_table(ctx->Md, mesh->n_plies, q.data());
+    chk(cudaMemcpyAsync(P.ply_q, q.data(), sizeof(q[0]) * q.size(), cudaMemcpyHostToDevice, ctx->stream));
+    if (all_boxes) chk(launch_box_records(D, box, ctx->stream));
+  };
   if (fp64) {
     wire(ctx->Dd, double{});
-    std::vector<double> q((size_t)kPlyStride<double> * mesh->n_plies);
-    ply_table(ctx->Md, mesh->n_plies, q.data());
-    chk(up(P.ply_q, q.data(), sizeof(double) * q.size()));
-    if (all_boxes) chk(launch_box_records(ctx->Dd, reinterpret_cast<double4_32a *>(P.box), ctx->stream));
+    up_table(ply_q64, ctx->Dd, reinterpret_cast<double4_32a *>(P.box));
   } else {
     wire(ctx->Df, float{});
-    std::vector<float> q((size_t)kPlyStride<float> * mesh->n_plies);
-    ply_table(ctx->Md, mesh->n_plies, q.data());
-    chk(up(P.ply_q, q.data(), sizeof(float) * q.size()));
-    if (all_boxes) chk(launch_box_records(ctx->Df, reinterpret_cast<float4 *>(P.box), ctx->stream));
+    up_table(ply_q32, ctx->Df, reinterpret_cast<float4 *>(P.box));
   }
   if (e != cudaSuccess) return die(PDN_E_CUDA, std::string("ply and box tables: ") + cudaGetErrorString(e));
   ctx->rmark_e_buf = d_rmark_e;

@@ -1,0 +1,46 @@
+"""A context on a stream that does not block on the default stream (any torch
+side stream): nothing orders the two, so every upload the kernels read has to
+be complete or on the context's own stream.  Whole runs equal those on the
+library's own stream bit for bit (the same kernels in the same order)."""
+import numpy as np
+import pytest
+
+import pdn_inputs as pi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import paper_2301_05552_gb300 as p
+    p.lib()
+    return p
+
+
+def _plate(nx, ny, plies, fp64, skew=False):
+    w = pi.damage_fp32_plate(nx=nx, ny=ny, plies=plies, Lx=0.5 * nx, Ly=0.5 * ny, H=0.275 * plies, fp64=fp64)
+    if skew:
+        Lx, Ly, _ = w.plate.dims
+        x, y = w.plate.X[0].copy(), w.plate.X[1].copy()
+        bump = np.sin(np.pi * x / Lx) * np.sin(np.pi * y / Ly)
+        w.plate.X[0] = x + 0.1 * bump * np.sin(9.0 * y / Ly)
+        w.plate.X[1] = y + 0.1 * bump * np.cos(7.0 * x / Lx)
+    return w
+
+
+@pytest.mark.parametrize("fp64,skew", [(True, False), (False, False), (False, True)])
+def test_created_and_stepped_on_a_side_stream(pkg, monkeypatch, fp64, skew):
+    import torch
+    monkeypatch.setenv("PDN_HEX_VARIANT", "0")
+    out = []
+    for stream in (None, torch.cuda.Stream().cuda_stream):
+        # a context with other ply angles first: its table is what a late
+        # upload would leave in reused memory
+        pkg.Solver(_plate(13, 9, 6, fp64, skew), stream=stream).close()
+        s = pkg.Solver(_plate(33, 27, 4, fp64, skew), stream=stream)
+        s.step(2000)  # contact after about 1,000
+        out.append(s.state()[:2] + pkg.pdn_get_contact(s.ctx))
+        s.close()
+    assert np.abs(out[0][0]).max() > 0.0
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
