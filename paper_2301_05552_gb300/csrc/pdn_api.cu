@@ -1663,8 +1663,10 @@ static int pdn_set_state_body(pdn_ctx *ctx, const double *d, const double *v) {
       }
   double *const *dd = ctx->precision == PDN_FP64 ? ctx->Dd.d : ctx->Df.d;
   double *const *vv = ctx->precision == PDN_FP64 ? ctx->Dd.v : ctx->Df.v;
-  PDN_CU(cudaMemcpy(dd[b], dh.data(), sizeof(double) * 3 * nn, cudaMemcpyHostToDevice), "write d");
-  PDN_CU(cudaMemcpy(vv[b], vh.data(), sizeof(double) * 3 * nn, cudaMemcpyHostToDevice), "write v");
+  // on the context's stream, where the kernels below read them (prime_state
+  // waits for the stream, so dh and vh outlive the copies)
+  PDN_CU(cudaMemcpyAsync(dd[b], dh.data(), sizeof(double) * 3 * nn, cudaMemcpyHostToDevice, ctx->stream), "write d");
+  PDN_CU(cudaMemcpyAsync(vv[b], vh.data(), sizeof(double) * 3 * nn, cudaMemcpyHostToDevice, ctx->stream), "write v");
   if (ctx->precision == PDN_FP64)
     k_mirror<double4_32a><<<grid_of(nn, 256), 256, 0, ctx->stream>>>(dd[b], ctx->Dd.u4[b], nn);
   else

@@ -44,3 +44,24 @@ def test_created_and_stepped_on_a_side_stream(pkg, monkeypatch, fp64, skew):
     assert np.abs(out[0][0]).max() > 0.0
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+def test_state_installed_on_a_side_stream(pkg, monkeypatch, fp64):
+    import torch
+    monkeypatch.setenv("PDN_HEX_VARIANT", "0")
+    w = _plate(65, 49, 8, fp64)  # 42,900 nodes: copies of a megabyte, several staging buffers each
+    Lx, Ly, _ = w.plate.dims
+    states = [pi.seeded_state(w.plate, k, amp=0.02, vamp=300.0, dimple=(0.5 * Lx, 0.5 * Ly, 0.12, 3.0)) for k in (7, 8)]
+    out = []
+    for stream in (None, torch.cuda.Stream().cuda_stream):
+        s = pkg.Solver(w, stream=stream)
+        got = []
+        for d, v in states:  # the second over the first's leftovers
+            pkg.pdn_set_state(s.ctx, d, v)
+            got += [pkg.pdn_internal_force(s.ctx), pkg.pdn_get_acceleration(s.ctx)]
+        s.step(40)
+        out.append(got + list(s.state()[:2]))
+        s.close()
+    for a, b in zip(*out):
+        assert np.abs(a).max() > 0.0 and np.array_equal(a, b)
