@@ -475,7 +475,9 @@ int build_tiles(pdn_batch *b, int tile_items) {
     const pdn_ctx *c = b->plates[p];
     nt[p] = make_int4(tiles(c->ns), tiles(c->nh) + tiles(coh_items(b, p)), tiles(c->nn), 1);
   }
-  PB_CU(cudaMemcpy(b->d_ntiles, nt.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice), "upload tile counts");
+  // on the batch's stream, where its kernels read them
+  PB_CU(cudaMemcpyAsync(b->d_ntiles, nt.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice, b->stream),
+        "upload tile counts");
   if (t.size() > b->tiles_cap) {
     if (b->d_tiles) cudaFree(b->d_tiles);
     b->d_tiles = nullptr;
@@ -483,7 +485,9 @@ int build_tiles(pdn_batch *b, int tile_items) {
     PB_CU(cudaMalloc(&b->d_tiles, sizeof(int4) * t.size()), "tile list");
     b->tiles_cap = t.size();
   }
-  PB_CU(cudaMemcpy(b->d_tiles, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice), "upload tiles");
+  PB_CU(cudaMemcpyAsync(b->d_tiles, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice, b->stream),
+        "upload tiles");
+  PB_CU(cudaStreamSynchronize(b->stream), "upload tiles");  // before t and nt go
   b->tile_items = tile_items;
   return PDN_OK;
 }
@@ -718,8 +722,12 @@ int upload_records(pdn_batch *b) {
   }
   PB_CU(cudaMalloc(&b->d_dev, sizeof(Dev<T>) * b->n), "plate records");
   PB_CU(cudaMalloc(&b->d_mat, sizeof(Mat<T>) * b->n), "plate materials");
-  PB_CU(cudaMemcpy(b->d_dev, D.data(), sizeof(Dev<T>) * b->n, cudaMemcpyHostToDevice), "upload plate records");
-  PB_CU(cudaMemcpy(b->d_mat, M.data(), sizeof(Mat<T>) * b->n, cudaMemcpyHostToDevice), "upload plate materials");
+  // on the batch's stream, where its kernels read them
+  PB_CU(cudaMemcpyAsync(b->d_dev, D.data(), sizeof(Dev<T>) * b->n, cudaMemcpyHostToDevice, b->stream),
+        "upload plate records");
+  PB_CU(cudaMemcpyAsync(b->d_mat, M.data(), sizeof(Mat<T>) * b->n, cudaMemcpyHostToDevice, b->stream),
+        "upload plate materials");
+  PB_CU(cudaStreamSynchronize(b->stream), "upload plate records");  // before D and M go
   return PDN_OK;
 }
 
@@ -813,7 +821,8 @@ static int pdn_batch_init_body(pdn_batch **out, int32_t n_plates, const pdn_mesh
       cudaMalloc(&b->d_ctl_all, sizeof(Ctl) * (size_t)n_plates + sizeof(BatchSync)) != cudaSuccess ||
       cudaMallocHost(&b->h_buf, sizeof(Ctl) * (size_t)n_plates + sizeof(BatchSync)) != cudaSuccess)
     return fail_init(PDN_E_OOM, "batch control buffers");
-  cudaMemset(b->d_sync, 0, sizeof(BatchSync));
+  const cudaError_t e = cudaMemsetAsync(b->d_sync, 0, sizeof(BatchSync), b->stream);
+  if (e != cudaSuccess) return fail_init(PDN_E_CUDA, std::string("batch control buffers: ") + cudaGetErrorString(e));
   *out = b;
   return PDN_OK;
 }

@@ -65,3 +65,26 @@ def test_state_installed_on_a_side_stream(pkg, monkeypatch, fp64):
         s.close()
     for a, b in zip(*out):
         assert np.abs(a).max() > 0.0 and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("schedule", ["0,0", "1,0"])
+def test_batch_on_a_side_stream(pkg, monkeypatch, schedule):
+    """Plate records, tile lists (one per candidate tile size while the batch
+    is tuned) and counters uploaded for the batch's stream, its own (which
+    never blocks on the default stream) or the caller's."""
+    import torch
+    monkeypatch.setenv("PDN_BATCH_SCHEDULE", schedule)
+    ws = [_plate(33, 27, 4, False), _plate(13, 9, 6, False), _plate(21, 40, 8, False)]
+    out = []
+    for stream in (None, torch.cuda.Stream().cuda_stream):
+        b = pkg.pdn_batch_init([w.plate for w in ws], [w.material for w in ws], stream=stream)
+        for w, ctx in zip(ws, b.plates):
+            Lx, Ly, _ = w.plate.dims
+            pkg.pdn_set_impactor(ctx, *w.impactor())
+            pkg.pdn_set_state(ctx, *pi.seeded_state(w.plate, 7, amp=0.02, vamp=300.0,
+                                                    dimple=(0.5 * Lx, 0.5 * Ly, 0.12, 1.5)))
+        pkg.pdn_batch_step(b, 100)
+        out.append([x for ctx in b.plates for x in pkg.pdn_get_state(ctx)[:2]])
+        b.close()
+    for a, c in zip(*out):
+        assert np.abs(a).max() > 0.0 and np.array_equal(a, c)
