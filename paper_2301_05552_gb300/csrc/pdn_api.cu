@@ -164,43 +164,6 @@ static int prime_state(pdn_ctx *ctx) {
   return PDN_OK;
 }
 
-// Bound on the strain components below which no point with the initial
-// history yields or reaches a damage onset (Mat::e_tol).  With every normal
-// component and engineering shear at most t, the tensor's Frobenius norm n is
-// at most sqrt(4.5) t, the same in ply axes, and each criterion of Algorithm 4
-// is bounded by a function of n: |e_ii| <= n; the 12, 13 shears together at
-// most sqrt(2) n; |sigma_ii| at most the norm of the stiffness row times n.
-// With the smallest seeded strengths and 0.1 % to spare for the rounding of
-// the criteria; unbounded when both laws are off.
-double elastic_strain_bound(const pdn_material &m, const double (&C)[3][3], double kT, int damage_on,
-                            int plasticity_on) {
-  double n = 1e30;
-  if (plasticity_on) n = std::min(n, m.Sp / (m.G12 * std::sqrt(2.0)));
-  if (damage_on) {
-    const double lo = 1.0 - std::fabs(m.spread);
-    const double r1 = std::sqrt(C[0][0] * C[0][0] + C[0][1] * C[0][1] + C[0][2] * C[0][2]);
-    const double r2 = std::sqrt(C[0][1] * C[0][1] + C[1][1] * C[1][1] + C[1][2] * C[1][2]);
-    n = std::min(n, std::min(m.XT * lo / m.E1, m.XC / r1));
-    const double a0 = m.alpha0_deg * M_PI / 180.0;
-    const double ST = m.YC * std::cos(a0) * (std::sin(a0) + std::cos(a0) / std::tan(2.0 * a0));
-    const double g = m.GYT / m.GSL, sl = std::sqrt(2.0) * std::max(m.G12, m.G13) / (m.SL * lo);
-    const double sq = std::sqrt(2.0) * m.G23 / ST, st = r2 * kT / ST, yt = r2 / (m.YT * lo);
-    auto matrix = [&](double x) {  // largest of the two matrix criteria at norm x
-      const double sh = (sl * sl + sq * sq) * x * x;
-      return std::max(std::fabs(1.0 - g) * yt * x + std::fabs(g) * yt * yt * x * x + sh, st * st * x * x + sh);
-    };
-    double hi = n, b = 0.0;
-    for (int k = 0; k < 200; ++k) {
-      const double mid = 0.5 * (b + hi);
-      if (matrix(mid) <= 1.0) b = mid;
-      else hi = mid;
-    }
-    n = b;
-  }
-  const double t = 0.999 * n / std::sqrt(4.5);
-  return t > 0.0 && std::isfinite(t) ? t : 0.0;
-}
-
 // Material constants in precision T from the double-precision record.
 template <typename T>
 int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_plies, int damage_on,
@@ -280,7 +243,8 @@ int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_pl
   M.eta = (T)m.eta;
   M.onset_floor = (T)(0.999 * std::min(KI * D3o * D3o, Ksh * Dsho * Dsho));
   M.spread = (T)m.spread;
-  M.e_tol = (T)elastic_strain_bound(m, C, ca * (sa + ca / t2), damage_on, plasticity_on);
+  M.e_tol = (T)elastic_strain_bound(m, C, damage_on, plasticity_on);
+  M.onset = onset_screen(m, C, damage_on, plasticity_on);
   M.seed = m.seed;
   M.damage_on = damage_on;
   M.plasticity_on = plasticity_on;

@@ -16,10 +16,15 @@
 // global axes (Dev::ply_q, 13 constants) without rotations.  The forces of
 // direction k need only sums of P_k over the pairs of points along k (four
 // values per component), in which du/dX_k is a common factor.  The test for
-// "cannot yield or damage" is one bound on the strain components
-// (Mat::e_tol, derived on the host from all criteria with the smallest seeded
-// strengths); elements it does not clear, or with history, are evaluated by
-// hex_lanes8, four at a time by the whole warp.
+// "cannot yield or damage" has two stages (pdn_screen.h): one bound on all
+// strain components (Mat::e_tol), then the criteria on the largest magnitude of
+// each component over the element's points.  Elements neither clears, or with
+// history, are evaluated by hex_lanes8, four at a time by the whole warp, which
+// costs about as much as the elastic form for all 32.  GB300, the point-by-point
+// kernel's time, the first stage alone, both: 24 plates in a batch late in their
+// impacts (up to 40 % of a plate's hexes past the first stage, 1 % damaged) 236,
+// 250, 166 us per step; the AS4/8552 coupon at 60,000 to 82,000 steps 87.1, 87.5,
+// 78.3 us, at its start, where the first stage clears all, 56.9, 41.2, 40.8 us.
 //
 // Every operation here is rounded explicitly (rmul, radd, rfma), so the
 // kernels that inline this code give the same bits.
@@ -38,6 +43,8 @@ __device__ __forceinline__ double rfma(double a, double b, double c) { return __
 
 // Magnitude as integer bits (the upper word of a double): compares as |x|
 // does, and a NaN compares above every finite bound.  Costs no FP64 work.
+// (max_mag below, of floats, drops a NaN: an element with a NaN strain may pass
+// as elastic; its forces are NaN either way, and the law would leave its history.)
 __device__ __forceinline__ uint32_t mag_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 __device__ __forceinline__ uint32_t mag_bits(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
@@ -349,6 +356,25 @@ __device__ __forceinline__ void hex_lanes8_item(const Dev<T> &D, const Mat<T> &M
 
 // ---------------------------------------------------------------------------
 // One thread per element: boxes that stay elastic (see the head of the file).
+// Largest magnitude of each strain component (xx yy zz | xy xz yz, engineering
+// shears) over an element's points: FP32 values, or upper words of doubles.
+template <typename T>
+struct StrainMag;
+template <>
+struct StrainMag<float> {
+  float m[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  __device__ __forceinline__ uint32_t largest() const {
+    return mag_bits(fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(m[4], m[5])));
+  }
+  __device__ __forceinline__ float upper(int k) const { return m[k]; }
+};
+template <>
+struct StrainMag<double> {
+  uint32_t m[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+  __device__ __forceinline__ uint32_t largest() const { return max(max(max(m[0], m[1]), max(m[2], m[3])), max(m[4], m[5])); }
+  __device__ __forceinline__ float upper(int k) const { return upper_float(m[k]); }
+};
+
 // Trilinear modes of the nodal displacements, unscaled (8 times the modes of
 // to_modes), by bin: bit 0 xi, bit 1 eta, bit 2 zeta.  V: float, double or a
 // packed pair of components.
@@ -433,13 +459,13 @@ __device__ __forceinline__ void column_sums(T g00, T g01, T g10, T g11, T t, T t
 }
 
 // FP64: nodal forces f (by node) of a box from its node displacements u (by
-// node), the box record {1/hx, 1/hy, 1/hz, volume/8} and the ply's constants;
-// returns the largest magnitude (mag_bits) of the strain components.  About
+// node), the box record {1/hx, 1/hy, 1/hz, volume/8} and the ply's constants,
+// and the largest magnitudes of the strain components.  About
 // 900 FP64 operations, against about 2,500 point by point; on this part an
 // FP64 operation holds a scheduler's pipe for 64 cycles, so they are the whole
 // cost.
-__device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], const double4_32a &box, const double *qp,
-                                                    double (&f)[8][3]) {
+__device__ __forceinline__ void hex_box_elastic(const double (&u)[8][3], const double4_32a &box, const double *qp,
+                                                double (&f)[8][3], StrainMag<double> &big) {
   const double gp = gauss_pt<double>();
   const double ih[3] = {box.x, box.y, box.z};
   double H0[3][2][2], H1[3][2][2], H2[3][2][2];  // [i][eta][zeta], [i][xi][zeta], [i][xi][eta]
@@ -473,7 +499,6 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
     return rfma(0.5, rfma(H[0][m][n], H[0][m][n], rfma(H[1][m][n], H[1][m][n], rmul(H[2][m][n], H[2][m][n]))),
                 H[k][m][n]);
   };
-  uint32_t big = 0;
   double E0[2][2], E1[2][2];
 #pragma unroll
   for (int m = 0; m < 2; ++m)
@@ -481,7 +506,8 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
     for (int n = 0; n < 2; ++n) {
       E0[m][n] = normal(H0, 0, m, n);
       E1[m][n] = normal(H1, 1, m, n);
-      big = max(big, max(mag_bits(E0[m][n]), mag_bits(E1[m][n])));
+      big.m[0] = max(big.m[0], mag_bits(E0[m][n]));
+      big.m[1] = max(big.m[1], mag_bits(E1[m][n]));
     }
   double G0[3][2][2], G1[3][2][2], G2[3][2][2], T0[2][2], T1[2][2], T2[2][2];
 #pragma unroll
@@ -489,7 +515,7 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
 #pragma unroll
     for (int ix = 0; ix < 2; ++ix) {
       const double e2 = normal(H2, 2, ix, iy);
-      big = max(big, mag_bits(e2));
+      big.m[2] = max(big.m[2], mag_bits(e2));
 #pragma unroll
       for (int iz = 0; iz < 2; ++iz) {
         const double a[3] = {H0[0][iy][iz], H0[1][iy][iz], H0[2][iy][iz]};
@@ -498,7 +524,9 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
         const double g01 = rfma(a[0], b[0], rfma(a[1], b[1], rfma(a[2], b[2], radd(a[1], b[0]))));
         const double g02 = rfma(a[0], d[0], rfma(a[1], d[1], rfma(a[2], d[2], radd(a[2], d[0]))));
         const double g12 = rfma(b[0], d[0], rfma(b[1], d[1], rfma(b[2], d[2], radd(b[2], d[1]))));
-        big = max(big, max(mag_bits(g01), max(mag_bits(g02), mag_bits(g12))));
+        big.m[3] = max(big.m[3], mag_bits(g01));
+        big.m[4] = max(big.m[4], mag_bits(g02));
+        big.m[5] = max(big.m[5], mag_bits(g12));
         const double e0 = E0[iy][iz], e1 = E1[ix][iz];
         const double S00 = rfma(c[0], e0, rfma(c[1], e1, rfma(c[2], e2, rmul(c[3], g01))));
         const double S11 = rfma(c[1], e0, rfma(c[4], e1, rfma(c[5], e2, rmul(c[6], g01))));
@@ -558,7 +586,6 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
 #pragma unroll
     for (int a = 0; a < 8; ++a) f[a][i] = C[bin_of(a)];
   }
-  return big;
 }
 
 // FP32, the same sums with the packed FP32 operations (two lanes per
@@ -570,8 +597,8 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const double (&u)[8][3], con
 __device__ __forceinline__ float lane_sum(float2 v) { return __fadd_rn(v.x, v.y); }
 __device__ __forceinline__ float max_mag(float m, float2 v) { return fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))); }
 
-__device__ __forceinline__ uint32_t hex_box_elastic(const float (&u)[8][3], const float4 &box, const float *qp,
-                                                    float (&f)[8][3]) {
+__device__ __forceinline__ void hex_box_elastic(const float (&u)[8][3], const float4 &box, const float *qp,
+                                                float (&f)[8][3], StrainMag<float> &big) {
   const float gp = gauss_pt<float>();
   const float ih[3] = {box.x, box.y, box.z};
   float2 H0[3][2], H1[3][2];  // [i][eta], [i][xi]; lanes zeta
@@ -631,13 +658,13 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const float (&u)[8][3], cons
     c[k + 1] = make_float2(v.z, v.w);
   }
   const float2 half = p2(0.5f);
-  float big = 0.0f;
   float2 E0[2], E1[2];
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
     E0[m] = pfma(half, pfma(H0[0][m], H0[0][m], pfma(H0[1][m], H0[1][m], pmul(H0[2][m], H0[2][m]))), H0[0][m]);
     E1[m] = pfma(half, pfma(H1[0][m], H1[0][m], pfma(H1[1][m], H1[1][m], pmul(H1[2][m], H1[2][m]))), H1[1][m]);
-    big = max_mag(max_mag(big, E0[m]), E1[m]);
+    big.m[0] = max_mag(big.m[0], E0[m]);
+    big.m[1] = max_mag(big.m[1], E1[m]);
   }
   float2 G0[3][2], G1[3][2], T0[2], T1[2];
   float G2[3][2][2];
@@ -647,13 +674,15 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const float (&u)[8][3], cons
     for (int ix = 0; ix < 2; ++ix) {
       const float d0 = H2[0][ix][iy], d1 = H2[1][ix][iy], d2 = H2[2][ix][iy];
       const float e2 = rfma(0.5f, rfma(d0, d0, rfma(d1, d1, rmul(d2, d2))), d2);
-      big = fmaxf(big, fabsf(e2));
+      big.m[2] = fmaxf(big.m[2], fabsf(e2));
       const float2 a[3] = {H0[0][iy], H0[1][iy], H0[2][iy]}, b[3] = {H1[0][ix], H1[1][ix], H1[2][ix]};
       const float2 d[3] = {p2(d0), p2(d1), p2(d2)};
       const float2 g01 = pfma(a[0], b[0], pfma(a[1], b[1], pfma(a[2], b[2], padd(a[1], b[0]))));
       const float2 g02 = pfma(a[0], d[0], pfma(a[1], d[1], pfma(a[2], d[2], padd(a[2], d[0]))));
       const float2 g12 = pfma(b[0], d[0], pfma(b[1], d[1], pfma(b[2], d[2], padd(b[2], d[1]))));
-      big = max_mag(max_mag(max_mag(big, g01), g02), g12);
+      big.m[3] = max_mag(big.m[3], g01);
+      big.m[4] = max_mag(big.m[4], g02);
+      big.m[5] = max_mag(big.m[5], g12);
       const float2 e0 = E0[iy], e1 = E1[ix], ez = p2(e2);
       const float2 S00 = pfma(c[0], e0, pfma(c[1], e1, pfma(c[2], ez, pmul(c[3], g01))));
       const float2 S11 = pfma(c[1], e0, pfma(c[4], e1, pfma(c[5], ez, pmul(c[6], g01))));
@@ -708,7 +737,6 @@ __device__ __forceinline__ uint32_t hex_box_elastic(const float (&u)[8][3], cons
 #pragma unroll
     for (int a = 0; a < 8; ++a) f[a][i] = C[bin_of(a)];
   }
-  return mag_bits(big);
 }
 
 // The lanes-of-eight evaluation kept out of line for the one-thread form's
@@ -762,8 +790,13 @@ __device__ __forceinline__ bool hex_box_pairs_core(const Dev<T> &D, const Mat<T>
     u[a][1] = v.y;
     u[a][2] = v.z;
   }
-  const uint32_t big = hex_box_elastic(u, box, D.ply_q + (int64_t)kPlyStride<T> * ply, f);
-  const bool ok = pristine && big < mag_bits(M.e_tol);
+  StrainMag<T> big;
+  hex_box_elastic(u, box, D.ply_q + (int64_t)kPlyStride<T> * ply, f, big);
+  bool ok = pristine && big.largest() < mag_bits(M.e_tol);
+  if (pristine && !ok) {
+    const float a[6] = {big.upper(0), big.upper(1), big.upper(2), big.upper(3), big.upper(4), big.upper(5)};
+    ok = clear_of_onset(M.onset, (float)M.ply_c[ply], (float)M.ply_s[ply], a);
+  }
   if (valid && ok) D.pflag[hb ^ 1][ee] = 1;
   uint32_t bad = __ballot_sync(kAll, valid && !ok);
   while (bad != 0u) {

@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "pdn_screen.h"
+
 namespace pdn {
 
 // Contact-surface nodes per block of the contact kernel, and per run of the
@@ -94,8 +96,10 @@ struct Mat {
   T spread;
   // every strain component (tensor normals, engineering shears, in any axes
   // about z) of magnitude below e_tol: no yield and no damage onset from the
-  // initial history, whatever the seeded strengths (the hex kernel's screen)
+  // initial history, whatever the seeded strengths (the hex kernel's first
+  // screen); the second is clear_of_onset (pdn_screen.h)
   T e_tol;
+  OnsetScreen onset;
   T ply_c[kMaxPlies], ply_s[kMaxPlies];
   uint64_t seed;
   int32_t damage_on, plasticity_on;
