@@ -160,13 +160,17 @@ typedef struct {
   int64_t device_bytes;    /* device memory held by the context */
   int32_t status;          /* sticky device status (PDN_OK or an error code) */
   int32_t precision;
-  int32_t hex_variant;     /* element-kernel launch variant chosen by the autotuner:
-                              0..3 hex kernel (interface kernel on a forked stream)
-                              with an occupancy target of 4, 5, 6 or 3 blocks/SM;
-                              4..7 one mixed hex + interface kernel with the same
-                              targets (never chosen by the autotuner, which times
-                              0..3).  The environment variable PDN_HEX_VARIANT
-                              (0..7) fixes it instead (no timing, tune_ms 0) */
+  int32_t hex_variant;     /* element-kernel launch variant.  FP32 boxes without the
+                              learned law: 0 or 3, the hex kernel with a register
+                              budget of four or three blocks of 128 per SM, whichever
+                              the autotuner timed faster at the first pdn_step; one
+                              kernel, 0, in FP64, for general hexes and with the
+                              learned law (not timed).  The environment variable
+                              PDN_HEX_VARIANT (0..7, FP32) fixes the number instead (no
+                              timing, tune_ms 0): 1 and 2 run the kernels of 0; 4..7
+                              one mixed hex + interface launch for contexts with
+                              interface elements (coh_pairs 0), the kernels of 0
+                              otherwise */
   int32_t sweep;           /* 0: separate element, interface and gather kernels; 1, 2, 3:
                               the column sweep (FP32 box hexes, flat interfaces, a plate
                               layered as a full grid of columns) with tiles of 16 x 8,
@@ -198,9 +202,9 @@ typedef struct {
                               pdn_init_mesh */
   int32_t reserved;
   double tune_ms[12];      /* mean time of an internal-force pass with each variant when
-                              tuned (0 if not): entries 0..3 the hex variants with separate
-                              kernels, entry 8 the column sweep (0 where none was planned);
-                              the fastest is used.  Entries 4..7, 9..11 unused */
+                              tuned (0 if not): entries 0 and 3 the hex variants, entry 8
+                              the column sweep (0 where none was planned); the faster hex
+                              variant is used.  The other entries are 0 */
 } pdn_info;
 
 /* Create a context on the current CUDA device: validate and copy the mesh,

@@ -1384,25 +1384,24 @@ int pdn_set_impactor(pdn_ctx *ctx, double radius, double mass, const double cent
   return PDN_OK;
 }
 
-// Autotuner: times every hex-kernel variant on force-evaluation passes of the
+// Autotuner: times the hex kernel's variants on force-evaluation passes of the
 // committed state (no side effect on the simulation) and keeps the fastest.
-// The variants differ only in their register budget.  The assembler may
-// contract multiply-adds differently under another budget, so results can
-// differ at FP32 rounding between variants (measured: the 3-block variant on
-// the cut-down AS4 coupon, 2e-7 relative after 2,000 steps; the 5- and
-// 6-block variants equal the 4-block one bit for bit).  Runs once per context, before the step
-// graph is captured.
+// Variants 0 and 3 are the one-thread form of FP32 boxes with a register
+// budget of four and three blocks of 128 per SM; the assembler may contract
+// multiply-adds differently under another budget (measured on the cut-down
+// AS4 coupon: 2e-7 relative after 2,000 steps).  General hexes, boxes with the
+// learned law and FP64 have one kernel each, and nothing is timed.  Runs once
+// per context, before the step graph is captured.
 int autotune(pdn_ctx *ctx) {
   if (ctx->tuned) return PDN_OK;
   ctx->tuned = true;
-  // variants timed by default: the hex kernel's four occupancy targets with
-  // separate element and gather kernels, and the column sweep where it was
-  // planned (the mixed hex + interface kernel, 4..7, is selected only by
-  // PDN_HEX_VARIANT: it times well in the first passes but loses once damage
-  // spreads)
-  const int nvar = ctx->precision == PDN_FP64 ? 1 : 4;
-  const int nsel = ctx->precision == PDN_FP64 ? 1 : 8;
-  if (nvar == 1) return PDN_OK;
+  if (ctx->precision == PDN_FP64) return PDN_OK;
+  // the numbers PDN_HEX_VARIANT takes (launch_hex, launch_elem): 1 and 2 run
+  // the kernels of 0, 5 to 7 those of 4, one mixed hex + interface launch for
+  // contexts that keep interface elements, selected only so (it times well in
+  // the first passes but loses once damage spreads)
+  constexpr int nsel = 8;
+  const bool budgets = ctx->Df.all_boxes && ctx->Df.sur_params == nullptr;
   const Sweep *sw = ctx->Df.sweep;
   // the sweep is kept only on request (PDN_SWEEP=1): the internal-force pass
   // the autotuner times does not show the cost of the node update in a
@@ -1426,6 +1425,7 @@ int autotune(pdn_ctx *ctx) {
       return PDN_OK;
     }
   }
+  if (!budgets && !sw) return PDN_OK;  // one kernel: variant 0
   cudaEvent_t ev[2];
   for (int k = 0; k < 2; ++k) PDN_CU(cudaEventCreate(&ev[k]), "tune event");
   const int reps = 8;
@@ -1451,7 +1451,8 @@ int autotune(pdn_ctx *ctx) {
   int best = 0;
   float best_ms = 1e30f;
   ctx->Df.sweep = nullptr;
-  for (int v = 0; v < nvar; ++v) {
+  for (int v : {0, 3}) {
+    if (!budgets) break;
     ctx->Df.hex_variant = v;
     int rc = time_pass(ctx->tune_ms[v]);
     if (rc) return rc;

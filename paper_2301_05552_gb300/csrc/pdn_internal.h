@@ -224,10 +224,11 @@ struct Dev {
   // element-force slots: 1 = eight per node (slot 8 j + k holds the k-th
   // entry of node j's CSR row, the rest stay zero), 0 = CSR positions
   int32_t ell;
-  // launch configuration picked by the autotuner: hex occupancy variant
-  // (0: 4 blocks of 128 per SM, 1: 5, 2: 6, 3: 3).  The variants execute the
-  // same source; results can differ at FP32 rounding between variants (the
-  // assembler's multiply-add contraction depends on the register budget).
+  // launch configuration picked by the autotuner: hex occupancy variant of
+  // FP32 boxes (0: 4 blocks of 128 per SM, 3: 3; pdn_info.hex_variant has the
+  // other numbers).  The variants execute the same source; results can differ
+  // at FP32 rounding between variants (the assembler's multiply-add
+  // contraction depends on the register budget).
   int32_t hex_variant;
   // learned law (FP32 box elements only): the network's parameters followed
   // by its scaling (include/pdn_surrogate.h), or nullptr for the exact law;

@@ -474,7 +474,8 @@ inline int grid_of(int64_t n, int b) {
 }  // namespace
 
 // Element kernel variants (pdn_info.hex_variant): 0..3 separate element
-// kernels, 4..7 one mixed hex + interface launch.
+// kernels (0 to 2 the same, 3 another register budget for FP32 boxes), 4..7 one
+// mixed hex + interface launch (FP32).
 constexpr int kMixedVariant = 4;
 
 template <typename T>
