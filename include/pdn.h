@@ -241,8 +241,9 @@ int pdn_set_impactor(pdn_ctx *ctx, double radius, double mass, const double cent
  * PDN_FULL_REPEAT=1, read by pdn_init_mesh, makes repetitions evaluate every
  * element and node, with the same results.  The kernels of a pass are
  * launched with programmatic dependent launch (each waits for the previous
- * grid before reading); PDN_PDL=0, read once per process, launches them
- * plainly, with the same results.  Returns after the work has completed on
+ * grid before reading); PDN_PDL=0, read once per process, launches them, the
+ * learned law's kernel and those of its training plainly, with the same
+ * results.  Returns after the work has completed on
  * the stream.
  * Errors: PDN_E_STATE without a striker, PDN_E_NONFINITE,
  * PDN_E_RELEASE_LIMIT (both sticky), PDN_E_CUDA. */

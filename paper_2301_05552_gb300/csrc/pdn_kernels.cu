@@ -20,6 +20,7 @@
 #include "pdn.h"
 #include "pdn_device.cuh"
 #include "pdn_items.cuh"
+#include "pdn_launch.h"
 
 namespace pdn {
 namespace {
@@ -441,29 +442,11 @@ __global__ void k_damage_field(Dev<T> D, Mat<T> M, int which, float *out) {
   out[e] = (float)m;
 }
 
-// Launch on the pass's main stream, with the programmatic-dependency
-// attribute unless PDN_PDL=0.
-bool pdl_on() {
-  static const bool on = [] {
-    const char *e = std::getenv("PDN_PDL");
-    return !(e && e[0] == '0');
-  }();
-  return on;
-}
-
-template <typename... KArgs, typename... Args>
-void launch_k(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl_on() ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, k, args...);
+// Launch on the pass's main stream (pdn_launch.h); an error is left to the
+// cudaGetLastError that ends the pass.
+template <typename K, typename... Args>
+void launch_k(K k, int grid, int block, cudaStream_t s, const Args &...args) {
+  launch_pdl(k, grid, block, 0, s, args...);
 }
 
 inline int grid_of(int64_t n, int b) {

@@ -18,6 +18,7 @@
 #include "pdn_context.h"
 #include "pdn_device.cuh"
 #include "pdn_internal.h"
+#include "pdn_launch.h"
 #include "pdn_mlp.cuh"
 #include "pdn_surrogate.h"
 
@@ -828,17 +829,7 @@ thread_local std::string g_sur_error;
 namespace pdn {
 cudaError_t launch_hex_sur(const Dev<float> &D, const Mat<float> &M, cudaStream_t s) {
   const int64_t g = (D.nh + kHexSurBlock - 1) / kHexSurBlock;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(g < 1 ? 1 : g));
-  cfg.blockDim = dim3(kHexSurBlock);
-  cfg.dynamicSmemBytes = kHexSurSmem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_hex_sur, D, M);
+  return launch_pdl(k_hex_sur, g < 1 ? 1 : g, kHexSurBlock, kHexSurSmem, s, D, M);
 }
 }  // namespace pdn
 
@@ -918,18 +909,8 @@ int train_begin(pdn_surrogate *s, int64_t B, int64_t rows) {
 int train_step(pdn_surrogate *s, const Scaling &sc, const float *X, const float *T, int64_t n_rows, int64_t B,
                int random, uint64_t seed, float lr, float *grad_out, int64_t row) {
   const int64_t tiles = B / kChunk;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)tiles);
-  cfg.blockDim = dim3(kTrainThreads);
-  cfg.dynamicSmemBytes = sizeof(TrainSmem);
-  cfg.stream = s->stream;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  PS_CU(cudaLaunchKernelEx(&cfg, k_train_tile, (const TrainImage *)s->img, sc, X, T, n_rows, B, (int32_t)random, seed,
-                           s->partW, s->partB, s->loss_part + row * tiles, s->status_dev),
+  PS_CU(launch_pdl(k_train_tile, tiles, kTrainThreads, sizeof(TrainSmem), s->stream, s->img, sc, X, T, n_rows, B, random,
+                   seed, s->partW, s->partB, s->loss_part + row * tiles, s->status_dev),
         "train tiles");
   float bc1 = 1.0f, bc2 = 1.0f;
   if (lr > 0.0f) {
@@ -937,11 +918,8 @@ int train_step(pdn_surrogate *s, const Scaling &sc, const float *X, const float 
     bc1 = 1.0f - std::pow(0.9f, (float)s->adam_t);
     bc2 = 1.0f - std::pow(0.999f, (float)s->adam_t);
   }
-  cfg.gridDim = dim3((kNumParams + 127) / 128);
-  cfg.blockDim = dim3(128);
-  cfg.dynamicSmemBytes = 0;
-  PS_CU(cudaLaunchKernelEx(&cfg, k_train_update, s->params, s->m1, s->m2, grad_out, s->img, (const float *)s->partW,
-                           (const float *)s->partB, tiles, lr, bc1, bc2),
+  PS_CU(launch_pdl(k_train_update, (kNumParams + 127) / 128, 128, 0, s->stream, s->params, s->m1, s->m2, grad_out, s->img,
+                   s->partW, s->partB, tiles, lr, bc1, bc2),
         "update");
   return PDN_OK;
 }
