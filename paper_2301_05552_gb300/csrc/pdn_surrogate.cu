@@ -171,9 +171,10 @@ constexpr int kTrainThreads = 2 * kTcRows;
 constexpr uint32_t kTrainTmem = 512;
 constexpr uint32_t kColW4 = 128, kColW3 = 192, kColW2 = 256, kColW1 = 320;
 
-// Whether the tensor core finished phase `phase` of the barrier, the same in
-// every thread; a wait that gave up is repeated once for what is in flight.
-__device__ __forceinline__ bool train_wait(uint64_t *bar, uint32_t phase) {
+// Whether the tensor core or a bulk copy finished phase `phase` of the barrier,
+// the same in every thread; a wait that gave up is repeated once for what is in
+// flight, which must not land in the shared memory of a CTA that has returned.
+__device__ __forceinline__ bool cta_wait(uint64_t *bar, uint32_t phase) {
   const bool done = umma::mbar_wait(bar, phase, kMaxPolls);
   if (__syncthreads_or(!done)) {
     umma::mbar_wait(bar, phase, kMaxPolls);
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   umma::fence_after_sync();
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the weights of the previous update
   if (t == 0) umma::bulk_load(&S.W, img, (uint32_t)sizeof(TrainImage), &S.bar_load);
-  bool ok = train_wait(&S.bar_load, 0);
+  bool ok = cta_wait(&S.bar_load, 0);
   const uint32_t lane_base = S.tmem + ((uint32_t)(warp & 3) << 21);
   uint32_t phase = 0;
   float y[kOutPad];
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       issue_chain(A, Bw, L == 0 ? kInPad : kHid, L == 3 ? kOutPad : kHid, S.tmem + col);
       umma::mma_commit(&S.bar);
     }
-    ok = train_wait(&S.bar, phase);
+    ok = cta_wait(&S.bar, phase);
     phase ^= 1u;
     if (!ok) break;
     if (L < 3) {
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       }
     }
     bias_sum(L + 1, L & 1);
-    ok = train_wait(&S.bar, phase);
+    ok = cta_wait(&S.bar, phase);
     phase ^= 1u;
     if (!ok) break;
     float v[32];
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       umma::mma_commit(&S.bar);
     }
     bias_sum(0, 1);
-    ok = train_wait(&S.bar, phase);
+    ok = cta_wait(&S.bar, phase);
   }
   if (ok && (warp & 3) < 2) {
     // rows (outputs) 0..63 of dW are lanes 0..63: warps 0 and 1 write layers 2
@@ -643,8 +644,7 @@ __global__ void __launch_bounds__(kHexSurBlock, 4)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
-  bool tc_ok = umma::mbar_wait(&S.bar_load, 0, kMaxPolls);
-  tc_ok = !__syncthreads_or(!tc_ok);
+  bool tc_ok = cta_wait(&S.bar_load, 0);
   const int mode = ctl->mode;
   if (mode >= MODE_DONE) return;
   const Scaling &sc = S.I.sc;
