@@ -196,11 +196,20 @@ typedef struct {
                               the partner from the node id, 1 otherwise (a partner table).
                               0: interface elements (k_coh).  The environment
                               variable PDN_COH_PAIRS=0, read by pdn_init_mesh, keeps the
-                              interface elements.  With 2, a node of an interface layer
-                              owns 4 element-force slots instead of 8 (its interface
-                              elements write none), unless PDN_SLOTS_COMPACT=0 is set at
-                              pdn_init_mesh */
-  int32_t reserved;
+                              interface elements.  With 2 and slots (planes 0), a node of
+                              an interface layer owns 4 element-force slots instead of 8
+                              (its interface elements write none), unless
+                              PDN_SLOTS_COMPACT=0 is set at pdn_init_mesh */
+  int32_t planes;          /* where the element kernels leave nodal forces for the gather.
+                              0: slots, one vector per node and element.  1: planes, one
+                              per component and rank of a node's elements: FP32, at most
+                              eight elements per node, no column sweep, and at least
+                              three quarters of the hexes with each corner one node id
+                              after their predecessor's (a structured numbering with rows
+                              of four hexes or more along the fastest axis).  The same
+                              forces summed in the same order: the same bits.  The
+                              environment variable PDN_PLANES=0, read by pdn_init_mesh,
+                              keeps slots */
   double tune_ms[12];      /* mean time of an internal-force pass with each variant when
                               tuned (0 if not): entries 0 and 3 the hex variants, entry 8
                               the column sweep (0 where none was planned); the faster hex

@@ -938,8 +938,12 @@ static int pdn_init_mesh_body(pdn_ctx **out, const pdn_mesh_desc *mesh, const pd
   // sweep) where three quarters of the hexes have each corner one node id
   // after their predecessor's, as in a structured numbering (every element of
   // a row but its first): a warp's stores to a plane are then whole lines.
-  // Otherwise each would be 32 separate 4-byte stores, three times the
-  // 16-byte ones of the slots.  PDN_PLANES=0, read here, keeps the slots.
+  // PDN_PLANES=0, read here, keeps the slots.  GB300, us per step, slots against
+  // planes (3 M hexes with interfaces in rows of n, a share (n - 1)/n
+  // consecutive): n = 16: 402, 373; 4 (the line): 435, 413; 3: 453, 435; 2: 484,
+  // 474.  The line is on the safe side: below it a share does not say how far a
+  // warp's stores scatter (children of a divided hex are adjacent, none
+  // consecutive: hex kernel 141 against 162 us, gather 137 against 114).
   const char *pl = std::getenv("PDN_PLANES");
   bool planes = opt->precision == PDN_FP32_FORCE && ell && !sweep_on && !(pl && pl[0] == '0' && pl[1] == '\0');
   if (planes) {
@@ -1775,7 +1779,7 @@ int pdn_get_info(pdn_ctx *ctx, pdn_info *info) {
     const bool layered = (f64 ? ctx->Dd.pair_layer : ctx->Df.pair_layer) > 0;
     info->coh_pairs = pairs ? (layered ? 2 : 1) : 0;
   }
-  info->reserved = 0;
+  info->planes = (ctx->precision == PDN_FP32_FORCE && ctx->Df.fplane != nullptr) ? 1 : 0;
   for (int v = 0; v < 12; ++v) info->tune_ms[v] = ctx->tune_ms[v];
   return PDN_OK;
 }
