@@ -185,14 +185,12 @@ __device__ __forceinline__ bool contact_item(const Dev<T> &D, int64_t s, int mod
 
 // ---------------------------------------------------------------------------
 // Kernel 2: hex8 internal forces of an item (pdn_hex.cuh): boxes one element
-// per thread (the warp calls together), other hexes eight lanes per element.
-// One box per thread; the warp calls together.
+// per thread (the warp calls together), other hexes eight lanes per element, or
+// one thread in large FP32 launches.
+// The nodal forces f of hex e (nodes nd) where the gather finds them.
 template <typename T>
-__device__ __forceinline__ void hex_item_box_pairs(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode) {
+__device__ __forceinline__ void store_hex(const Dev<T> &D, int64_t e, const T (&f)[8][3]) {
   using V4 = typename Vec4T<T>::type;
-  T f[8][3];
-  int nd[8];
-  if (!hex_box_pairs_core(D, M, e, valid, mode, f, nd)) return;
   if constexpr (sizeof(T) == 4) {
     if (D.fplane != nullptr) {
       plane_store8(D, D.hex, e, e, f);
@@ -211,6 +209,28 @@ __device__ __forceinline__ void hex_item_box_pairs(const Dev<T> &D, const Mat<T>
     o.w = T(0);
     D.fe[ps[a]] = o;
   }
+}
+
+// One box per thread; the warp calls together.
+template <typename T>
+__device__ __forceinline__ void hex_item_box_pairs(const Dev<T> &D, const Mat<T> &M, int64_t e, bool valid, int mode) {
+  T f[8][3];
+  int nd[8];
+  if (hex_box_pairs_core(D, M, e, valid, mode, f, nd)) store_hex(D, e, f);
+}
+
+// One general hex per thread, point by point (FP32).
+__device__ __forceinline__ void hex_item_points(const Dev<float> &D, const Mat<float> &M, int64_t e, int mode) {
+  if (e >= D.nh) return;
+  if (mode == MODE_REPEAT && !repeat_take(D.rmark_e, e)) return;
+  const int4 c0 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e);
+  const int4 c1 = __ldg(reinterpret_cast<const int4 *>(D.hex) + 2 * e + 1);
+  const int nd[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+  if (!nodes_in_range(D, nd)) return;
+  if (mode == MODE_REPEAT) repeat_mark_nodes(D.rmark_n, nd);
+  float f[8][3];
+  hex_points(D, M, e, mode, nd, f);
+  store_hex(D, e, f);
 }
 
 template <typename T, bool BOX>

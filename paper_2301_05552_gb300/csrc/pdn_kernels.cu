@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(128, MINB) k_hex(const __grid_constant__ Dev<T
   hex_item_box_pairs(D, M, e, e < D.nh, mode);
 }
 
-// Eight lanes per element: general hexes, and boxes in launches too small to
-// fill the GPU with one thread per element.
+// Eight lanes per element: general hexes, and FP64 boxes in launches too small
+// to fill the GPU with one thread per element.
 template <typename T, bool BOX>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3)
     k_hex_lanes8(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M) {
@@ -72,6 +72,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3)
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
   hex_lanes8_item<T, BOX>(D, M, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, D.nh, mode);
+}
+
+// General FP32 hexes, one thread per element (launches from kPointsFrom hexes on).
+__global__ void __launch_bounds__(128, 4)
+    k_hex_points(const __grid_constant__ Dev<float> D, const __grid_constant__ Mat<float> M) {
+  pdl_enter();
+  const int mode = D.ctl->mode;
+  if (mode >= MODE_DONE) return;
+  hex_item_points(D, M, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, mode);
 }
 
 template <typename T, bool FLAT, int MINB>
@@ -475,13 +484,18 @@ void launch_elem(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
 // its scheduler 64 cycles whether one warp or more are resident, so the
 // launch takes (warps on the fullest scheduler) x (operations per warp): about
 // 900 per warp of 32 elements, or 170 per warp of 4.
-template <typename T>
-bool hex_lanes8_fits(const Dev<T> &D) {
-  if (sizeof(T) == 4) return false;
+inline bool hex_lanes8_fits(const Dev<double> &D) {
   const int64_t schedulers = 4 * 152;
   const int64_t w1 = (D.nh + 31) / 32, w8 = (D.nh + 3) / 4;
   return (w8 + schedulers - 1) / schedulers * 170 <= (w1 + schedulers - 1) / schedulers * 900;
 }
+
+// General FP32 hexes: one thread per element from two and a half rounds of its
+// four blocks per SM on, eight lanes below.  Lanes fill the GPU with an eighth of
+// the elements, but repeat the shuffles' work; GB300, lanes against one thread,
+// us per step: 98,304 hexes 35.9, 37.4; 145,800: 44.1, 45.3; 210,000: 72.5, 66.2;
+// 393,216: 131.8, 116.3; 3.84 M: 1,142, 991 (all damaged: 1,633, 1,167).
+constexpr int64_t kPointsFrom = 5 * 4 * 128 * 152 / 2;
 
 template <typename T>
 void launch_hex(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
@@ -490,17 +504,21 @@ void launch_hex(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
       launch_hex_sur(D, M, s);
       return;
     }
+    if (!D.all_boxes && D.nh >= kPointsFrom) {
+      launch_k(k_hex_points, grid_of(D.nh, 128), 128, s, D, M);
+      return;
+    }
   }
   if (!D.all_boxes)
     launch_k(k_hex_lanes8<T, false>, grid_of(8 * D.nh, 128), 128, s, D, M);
-  else if (hex_lanes8_fits(D))
-    launch_k(k_hex_lanes8<T, true>, grid_of(8 * D.nh, 128), 128, s, D, M);
   else if constexpr (std::is_same<T, float>::value) {
     const int g = grid_of(D.nh, 128);
     switch (D.hex_variant) {
       case 3: launch_k(k_hex<T, 3>, g, 128, s, D, M); break;
       default: launch_k(k_hex<T, 4>, g, 128, s, D, M); break;
     }
+  } else if (hex_lanes8_fits(D)) {
+    launch_k(k_hex_lanes8<T, true>, grid_of(8 * D.nh, 128), 128, s, D, M);
   } else {
     launch_k(k_hex<T, 2>, grid_of(D.nh, 128), 128, s, D, M);
   }
