@@ -66,3 +66,29 @@ def test_strained_boxes_match_oracle(pkg, nx, ny, plies, fp64, ramp):
     assert has_o.any() == ramp and not has_o.all()
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("nx,ny,plies", [(33, 13, 4), (39, 39, 8)])
+def test_plates_with_a_history_everywhere_match_oracle(pkg, nx, ny, plies, fp64):
+    """Warps without one pristine element: a plate sheared past yield takes 8
+    steps, and the force at its own state and history is the oracle's."""
+    w = _free_plate(nx, ny, plies, fp64)
+    x, y, z = w.plate.X
+    d = np.stack([-0.008 * x + 0.008 * y, 0.008 * x + 0.008 * y, -0.001 * z])
+    tol = 1e-10 if fp64 else 1e-4
+    g, o = pkg.Solver(w), oracle.model_for(w)
+    pkg.pdn_set_state(g.ctx, d, np.zeros_like(d))
+    o.set_state(d, np.zeros_like(d))
+    g.step(8)
+    assert o.step(8) == 0
+    hist, r = pkg.pdn_get_history(g.ctx)
+    h = hist.reshape(7, 8, -1)
+    assert ((h[:4] > 1.0).any((0, 1)) | (h[4:] != 0.0).any((0, 1))).all()
+    dg, vg, _ = g.state()
+    o.set_state(dg, vg)
+    o.set_history(hist.astype(np.float64).transpose(2, 1, 0), r.astype(np.float64).T)
+    fg, fo = pkg.pdn_internal_force(g.ctx), o.internal_force()
+    assert np.abs(fo).max() > 0.0 and np.abs(fg - fo).max() <= tol * np.abs(fo).max()
+    g.close()
+    o.close()
