@@ -53,14 +53,17 @@ __global__ void __launch_bounds__(kActRun) k_contact(const __grid_constant__ Dev
   if (D.act_cnt != nullptr && threadIdx.x == 0) D.act_cnt[blockIdx.x] = c;
 }
 
-// Boxes, one element per thread.
+// Boxes, one element per thread: the first 2^lanes_log2 lanes of each warp.
 template <typename T, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_hex(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M) {
+__global__ void __launch_bounds__(128, MINB)
+    k_hex(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M, int lanes_log2) {
   pdl_enter();
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  hex_item_box_pairs(D, M, e, e < D.nh, mode);
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = (int)(threadIdx.x & 31);
+  const int64_t e = (w << lanes_log2) + lane;
+  hex_item_box_pairs(D, M, e, lane >> lanes_log2 == 0 && e < D.nh, mode);
 }
 
 // Eight lanes per element: general hexes, and FP64 boxes in launches too small
@@ -490,6 +493,19 @@ inline bool hex_lanes8_fits(const Dev<double> &D) {
   return (w8 + schedulers - 1) / schedulers * 170 <= (w1 + schedulers - 1) / schedulers * 900;
 }
 
+// FP32 boxes per warp in small launches: 8 or 16 instead of 32 while there are no
+// more warps than half the schedulers, so that a warp whose elements all need
+// the point-by-point form goes two or four rounds instead of eight.  The same
+// bits.  GB300, 32 per warp against this, us per step, undamaged and damaged all
+// over (the former point-by-point kernel's time): 384 hexes 13.4, 13.3 and 36.7,
+// 21.3 (29.5); 1,536: 13.6, 13.6 and 36.3, 21.9 (30.1); 4,800: 13.6, 13.7 and
+// 32.5, 24.6 (28.1).  At 7,680 16 per warp cost the undamaged step 5 %.
+inline int hex_lanes_log2(int64_t nh) {
+  int lg = 3;
+  while (lg < 5 && ((nh - 1) >> lg) + 1 > 2 * 152) ++lg;
+  return lg;
+}
+
 // General FP32 hexes: one thread per element from two and a half rounds of its
 // four blocks per SM on, eight lanes below.  Lanes fill the GPU with an eighth of
 // the elements, but repeat the shuffles' work; GB300, lanes against one thread,
@@ -512,15 +528,15 @@ void launch_hex(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
   if (!D.all_boxes)
     launch_k(k_hex_lanes8<T, false>, grid_of(8 * D.nh, 128), 128, s, D, M);
   else if constexpr (std::is_same<T, float>::value) {
-    const int g = grid_of(D.nh, 128);
+    const int lg = hex_lanes_log2(D.nh), g = grid_of(D.nh, 4 << lg);
     switch (D.hex_variant) {
-      case 3: launch_k(k_hex<T, 3>, g, 128, s, D, M); break;
-      default: launch_k(k_hex<T, 4>, g, 128, s, D, M); break;
+      case 3: launch_k(k_hex<T, 3>, g, 128, s, D, M, lg); break;
+      default: launch_k(k_hex<T, 4>, g, 128, s, D, M, lg); break;
     }
   } else if (hex_lanes8_fits(D)) {
     launch_k(k_hex_lanes8<T, true>, grid_of(8 * D.nh, 128), 128, s, D, M);
   } else {
-    launch_k(k_hex<T, 2>, grid_of(D.nh, 128), 128, s, D, M);
+    launch_k(k_hex<T, 2>, grid_of(D.nh, 128), 128, s, D, M, 5);
   }
 }
 
