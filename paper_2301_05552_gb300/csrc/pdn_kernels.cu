@@ -97,10 +97,10 @@ __global__ void __launch_bounds__(128, MINB) k_coh(Dev<T> D, Mat<T> M) {
 // Hex and interface elements in one launch: blocks alternate between a tile
 // of hexes and a tile of interface elements (then the remainder of the
 // larger kind), so that every SM runs both the compute-bound hex warps and
-// the latency-bound interface warps at the same time.
-template <typename T, bool BOX, int MINB>
-__global__ void __launch_bounds__(128, MINB)
-    k_elem(const __grid_constant__ Dev<T> D, const __grid_constant__ Mat<T> M, int nbh, int nbc) {
+// the latency-bound interface warps at the same time (FP32, on request).
+template <bool BOX>
+__global__ void __launch_bounds__(128, 4)
+    k_elem(const __grid_constant__ Dev<float> D, const __grid_constant__ Mat<float> M, int nbh, int nbc) {
   pdl_enter();
   const int mode = D.ctl->mode;
   if (mode >= MODE_DONE) return;
@@ -115,11 +115,11 @@ __global__ void __launch_bounds__(128, MINB)
   }
   const int64_t first = (int64_t)idx * blockDim.x, i = first + threadIdx.x;
   if (kind == 0)
-    hex_item<T, BOX>(D, M, first, min(D.nh, first + (int64_t)blockDim.x), mode);
+    hex_item<float, BOX>(D, M, first, min(D.nh, first + (int64_t)blockDim.x), mode);
   else if (D.all_flat_coh)
-    coh_item<T, true>(D, M, i, mode);
+    coh_item<float, true>(D, M, i, mode);
   else
-    coh_item<T, false>(D, M, i, mode);
+    coh_item<float, false>(D, M, i, mode);
 }
 
 template <typename T>
@@ -473,14 +473,13 @@ inline int grid_of(int64_t n, int b) {
 // mixed hex + interface launch (FP32).
 constexpr int kMixedVariant = 4;
 
-template <typename T>
-void launch_elem(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
+inline void launch_elem(const Dev<float> &D, const Mat<float> &M, cudaStream_t s) {
   const int nbh = grid_of(D.nh, 128), nbc = D.nc > 0 ? (int)((D.nc + 127) / 128) : 0;
   const int g = nbh + nbc;
   if (D.all_boxes)
-    launch_k(k_elem<T, true, 4>, g, 128, s, D, M, nbh, nbc);
+    launch_k(k_elem<true>, g, 128, s, D, M, nbh, nbc);
   else
-    launch_k(k_elem<T, false, 4>, g, 128, s, D, M, nbh, nbc);
+    launch_k(k_elem<false>, g, 128, s, D, M, nbh, nbc);
 }
 
 // FP64 boxes: one thread per element or eight lanes.  An FP64 operation holds
@@ -598,8 +597,6 @@ cudaError_t launch_pass(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_
       return cudaGetLastError();
     }
   }
-  bool mixed = D.hex_variant >= kMixedVariant && D.ipair == nullptr;
-  if constexpr (std::is_same<T, float>::value) mixed = mixed && D.sur_params == nullptr;
   if (D.ipair != nullptr) {
     // interfaces as node pairs: no interface kernel; the interface event
     // pair is empty
@@ -618,19 +615,21 @@ cudaError_t launch_pass(const Dev<T> &D, const Mat<T> &M, cudaStream_t s, int32_
     if (ev) cudaEventRecord(ev[5], s);
     return cudaGetLastError();
   }
-  if (mixed) {
-    // one launch for both element kinds; the interface event pair is empty
-    if (ev) cudaEventRecord(ev[0], s);
-    launch_k(k_contact<T>, grid_of(D.ns, kActRun), kActRun, s, D);
-    if (ev) cudaEventRecord(ev[1], s);
-    launch_elem(D, M, s);
-    if (ev) cudaEventRecord(ev[2], s);
-    if (ev) cudaEventRecord(ev[3], s);
-    launch_k(k_gather<T>, grid_of(D.nn, gather_block), gather_block, s, D);
-    if (ev) cudaEventRecord(ev[4], s);
-    launch_k(k_tail<T>, 1, 256, s, D);
-    if (ev) cudaEventRecord(ev[5], s);
-    return cudaGetLastError();
+  if constexpr (std::is_same<T, float>::value) {
+    if (D.hex_variant >= kMixedVariant && D.sur_params == nullptr) {
+      // one launch for both element kinds; the interface event pair is empty
+      if (ev) cudaEventRecord(ev[0], s);
+      launch_k(k_contact<T>, grid_of(D.ns, kActRun), kActRun, s, D);
+      if (ev) cudaEventRecord(ev[1], s);
+      launch_elem(D, M, s);
+      if (ev) cudaEventRecord(ev[2], s);
+      if (ev) cudaEventRecord(ev[3], s);
+      launch_k(k_gather<T>, grid_of(D.nn, gather_block), gather_block, s, D);
+      if (ev) cudaEventRecord(ev[4], s);
+      launch_k(k_tail<T>, 1, 256, s, D);
+      if (ev) cudaEventRecord(ev[5], s);
+      return cudaGetLastError();
+    }
   }
   const bool concurrent = side != nullptr && ev == nullptr && D.nc > 0;
   if (ev) cudaEventRecord(ev[0], s);
