@@ -243,8 +243,8 @@ int fill_mat(Mat<T> &M, const pdn_material &m, const double *ply_angle, int n_pl
   M.eta = (T)m.eta;
   M.onset_floor = (T)(0.999 * std::min(KI * D3o * D3o, Ksh * Dsho * Dsho));
   M.spread = (T)m.spread;
-  M.e_tol = (T)elastic_strain_bound(m, C, damage_on, plasticity_on);
-  M.onset = onset_screen(m, C, damage_on, plasticity_on);
+  M.e_tol = (T)elastic_strain_bound(m, C, ca * (sa + ca / t2), damage_on, plasticity_on);
+  M.onset = onset_screen(m, C, ca * (sa + ca / t2), damage_on, plasticity_on);
   M.seed = m.seed;
   M.damage_on = damage_on;
   M.plasticity_on = plasticity_on;

@@ -45,19 +45,12 @@ struct OnsetScreen {
 };
 
 namespace screen {
-struct Limits {  // smallest seeded strengths
+struct Limits {  // smallest seeded strengths; kT = ca (sa - etaT ca) of Algorithm 4
   double XT, YT, SL, ST, kT, g;
 };
-inline Limits limits(const pdn_material &m) {
-  const double lo = 1.0 - std::fabs(m.spread), a0 = m.alpha0_deg * M_PI / 180.0;
-  Limits l;
-  l.XT = m.XT * lo;
-  l.YT = m.YT * lo;
-  l.SL = m.SL * lo;
-  l.kT = std::cos(a0) * (std::sin(a0) + std::cos(a0) / std::tan(2.0 * a0));
-  l.ST = m.YC * l.kT;
-  l.g = m.GYT / m.GSL;
-  return l;
+inline Limits limits(const pdn_material &m, double kT) {
+  const double lo = 1.0 - std::fabs(m.spread);
+  return {m.XT * lo, m.YT * lo, m.SL * lo, m.YC * kT, kT, m.GYT / m.GSL};
 }
 }  // namespace screen
 
@@ -68,53 +61,51 @@ inline Limits limits(const pdn_material &m) {
 // is bounded by a function of n: |e_ii| <= n; the 12, 13 shears together at
 // most sqrt(2) n; |sigma_ii| at most the norm of the stiffness row times n.
 // With the smallest seeded strengths and 0.1 % to spare for the rounding of
-// the criteria; unbounded when both laws are off.
-inline double elastic_strain_bound(const pdn_material &m, const double (&C)[3][3], int damage_on, int plasticity_on) {
+// the criteria; unbounded when both laws are off, 0 where a limit is no number.
+inline double elastic_strain_bound(const pdn_material &m, const double (&C)[3][3], double kT, int damage_on,
+                                   int plasticity_on) {
   double n = 1e30;
-  if (plasticity_on) n = std::min(n, m.Sp / (m.G12 * std::sqrt(2.0)));
+  auto cap = [&](double x) { n = x < n ? x : (x >= n ? n : 0.0); };
+  if (plasticity_on) cap(m.Sp / (m.G12 * std::sqrt(2.0)));
   if (damage_on) {
-    const screen::Limits l = screen::limits(m);
+    const screen::Limits l = screen::limits(m, kT);
     const double r1 = std::sqrt(C[0][0] * C[0][0] + C[0][1] * C[0][1] + C[0][2] * C[0][2]);
     const double r2 = std::sqrt(C[0][1] * C[0][1] + C[1][1] * C[1][1] + C[1][2] * C[1][2]);
-    n = std::min(n, std::min(l.XT / m.E1, m.XC / r1));
+    cap(l.XT / m.E1);
+    cap(m.XC / r1);
     const double sl = std::sqrt(2.0) * std::max(m.G12, m.G13) / l.SL;
     const double sq = std::sqrt(2.0) * m.G23 / l.ST, st = r2 * l.kT / l.ST, yt = r2 / std::fabs(l.YT);
-    auto matrix = [&](double x) {  // largest of the two matrix criteria at norm x
-      const double sh = (sl * sl + sq * sq) * x * x;
-      return std::max(std::fabs(1.0 - l.g) * yt * x + std::fabs(l.g) * yt * yt * x * x + sh, st * st * x * x + sh);
-    };
-    double hi = n, b = 0.0;
-    for (int k = 0; k < 200; ++k) {
-      const double mid = 0.5 * (b + hi);
-      if (matrix(mid) <= 1.0) b = mid;
-      else hi = mid;
-    }
-    n = b;
+    // the matrix criteria at norm x: |1 - g| yt x + (|g| yt^2 + sh) x^2 <= 1 and (st^2 + sh) x^2 <= 1
+    const double sh = sl * sl + sq * sq, q = std::fabs(l.g) * yt * yt + sh, p = std::fabs(1.0 - l.g) * yt;
+    cap(2.0 / (p + std::sqrt(p * p + 4.0 * q)));
+    cap(1.0 / std::sqrt(st * st + sh));
   }
   const double t = 0.999 * n / std::sqrt(4.5);
   return t > 0.0 && std::isfinite(t) ? t : 0.0;
 }
 
-inline OnsetScreen onset_screen(const pdn_material &m, const double (&C)[3][3], int damage_on, int plasticity_on) {
+inline OnsetScreen onset_screen(const pdn_material &m, const double (&C)[3][3], double kT, int damage_on,
+                                int plasticity_on) {
   OnsetScreen o{};
   // an upper bound in FP32; what is negative or no number clears nothing
   auto up = [](double v) { return v >= 0.0 && v < 1e30 ? (float)(v * (1.0 + 1e-6)) : INFINITY; };
   auto pos = [](double v) { return v > 0.0 ? v : NAN; };  // a strength that is none clears nothing
   if (damage_on) {
-    const screen::Limits l = screen::limits(m);
+    const screen::Limits l = screen::limits(m, kT);
+    const double iXC = 1.0 / pos(m.XC), iYT = 1.0 / pos(l.YT), iSL = 1.0 / pos(l.SL), iST = 1.0 / l.ST;
     o.ft = up(m.E1 / pos(l.XT));
-    o.fc1 = up(std::fabs(C[0][0]) / pos(m.XC));
-    o.fc2 = up(std::fabs(C[0][1]) / pos(m.XC));
-    o.fc3 = up(std::fabs(C[0][2]) / pos(m.XC));
-    o.y1 = up(std::fabs(C[0][1]) / pos(l.YT));
-    o.y2 = up(std::fabs(C[1][1]) / pos(l.YT));
-    o.y3 = up(std::fabs(C[1][2]) / pos(l.YT));
+    o.fc1 = up(std::fabs(C[0][0]) * iXC);
+    o.fc2 = up(std::fabs(C[0][1]) * iXC);
+    o.fc3 = up(std::fabs(C[0][2]) * iXC);
+    o.y1 = up(std::fabs(C[0][1]) * iYT);
+    o.y2 = up(std::fabs(C[1][1]) * iYT);
+    o.y3 = up(std::fabs(C[1][2]) * iYT);
     o.g1 = up(std::max(1.0 - l.g, 0.0));  // a negative term is left out
     o.g = up(l.g);
-    const double t = l.YT * std::max(l.kT, 0.0) / l.ST, s = m.G23 / l.ST;
+    const double t = l.YT * std::max(l.kT, 0.0) * iST, s = m.G23 * iST, s12 = m.G12 * iSL, s13 = m.G13 * iSL;
     o.mc2 = up(t * t);
-    o.h12 = up(m.G12 / pos(l.SL) * (m.G12 / l.SL));
-    o.h13 = up(m.G13 / pos(l.SL) * (m.G13 / l.SL));
+    o.h12 = up(s12 * s12);
+    o.h13 = up(s13 * s13);
     o.h23 = up(s * s);
   }
   if (plasticity_on) {

@@ -20,11 +20,15 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SRC = r"""
 #include "pdn_screen.h"
 using namespace pdn;
+static double kt(const pdn_material &m) {
+  const double a = m.alpha0_deg * M_PI / 180.0;
+  return std::cos(a) * (std::sin(a) + std::cos(a) / std::tan(2.0 * a));
+}
 extern "C" double bound(const pdn_material *m, const double (*C)[3], int dm, int pl) {
-  return elastic_strain_bound(*m, *reinterpret_cast<const double (*)[3][3]>(C), dm, pl);
+  return elastic_strain_bound(*m, *reinterpret_cast<const double (*)[3][3]>(C), kt(*m), dm, pl);
 }
 extern "C" int cleared(const pdn_material *m, const double (*C)[3], int dm, int pl, double c, double s, const float *a) {
-  const OnsetScreen o = onset_screen(*m, *reinterpret_cast<const double (*)[3][3]>(C), dm, pl);
+  const OnsetScreen o = onset_screen(*m, *reinterpret_cast<const double (*)[3][3]>(C), kt(*m), dm, pl);
   return clear_of_onset(o, (float)c, (float)s, *reinterpret_cast<const float (*)[6]>(a));
 }
 extern "C" float upper(uint32_t hi) { return upper_float(hi); }
