@@ -586,9 +586,9 @@ __global__ void k_init_params(float *p, uint64_t seed) {
 }
 
 // ---------------------------------------------------------------------------
-// Hex8 of an axis-aligned box (FP32) with the learned law where it applies.
-// Same formulation and arithmetic as the scalar element of pdn_items.cuh
-// (Eq. fcont, Algorithm 4); at each Gauss point the exact plasticity runs
+// Hex8 of an axis-aligned box (FP32) with the learned law where it applies, one
+// thread per element, point by point, through trilinear modes (Eq. fcont,
+// Algorithm 4; the formulation of hex_points in pdn_hex.cuh); at each Gauss point the exact plasticity runs
 // first, then either the network (all loading-function ratios at most the
 // context's onset ratio and every input inside the training box: the
 // thresholds do not change there) or the exact damage part.  The network
