@@ -954,12 +954,12 @@ def hex_sections(text: str) -> str:
 
 def kernel_source_hash() -> str:
     """Hash of the source k_hex is compiled from: the kernel file, the element
-    bodies, the device helpers and records, and the element sections of the
-    item bodies.  A
-    stored DRAM-traffic record of k_hex counts only while this matches."""
+    bodies and their screens, the device helpers and records, and the element
+    sections of the item bodies.  A stored DRAM-traffic record of k_hex counts
+    only while this matches."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("pdn_kernels.cu", "pdn_items.cuh", "pdn_hex.cuh", "pdn_device.cuh", "pdn_internal.h"):
+    for name in ("pdn_kernels.cu", "pdn_items.cuh", "pdn_hex.cuh", "pdn_screen.h", "pdn_device.cuh", "pdn_internal.h"):
         with open(os.path.join(ROOT, "paper_2301_05552_gb300", "csrc", name), encoding="utf-8") as f:
             text = f.read()
         if name == "pdn_items.cuh":

@@ -482,12 +482,16 @@ inline void launch_elem(const Dev<float> &D, const Mat<float> &M, cudaStream_t s
     launch_k(k_elem<false>, g, 128, s, D, M, nbh, nbc);
 }
 
+// SMs of a GB300.  The rules that use it choose between forms of the same
+// results: on another count they choose less well, not wrongly.
+constexpr int64_t kSms = 152;
+
 // FP64 boxes: one thread per element or eight lanes.  An FP64 operation holds
 // its scheduler 64 cycles whether one warp or more are resident, so the
 // launch takes (warps on the fullest scheduler) x (operations per warp): about
 // 900 per warp of 32 elements, or 170 per warp of 4.
 inline bool hex_lanes8_fits(const Dev<double> &D) {
-  const int64_t schedulers = 4 * 152;
+  const int64_t schedulers = 4 * kSms;
   const int64_t w1 = (D.nh + 31) / 32, w8 = (D.nh + 3) / 4;
   return (w8 + schedulers - 1) / schedulers * 170 <= (w1 + schedulers - 1) / schedulers * 900;
 }
@@ -501,7 +505,7 @@ inline bool hex_lanes8_fits(const Dev<double> &D) {
 // 32.5, 24.6 (28.1).  At 7,680 16 per warp cost the undamaged step 5 %.
 inline int hex_lanes_log2(int64_t nh) {
   int lg = 3;
-  while (lg < 5 && ((nh - 1) >> lg) + 1 > 2 * 152) ++lg;
+  while (lg < 5 && ((nh - 1) >> lg) + 1 > 2 * kSms) ++lg;
   return lg;
 }
 
@@ -510,7 +514,7 @@ inline int hex_lanes_log2(int64_t nh) {
 // the elements, but repeat the shuffles' work; GB300, lanes against one thread,
 // us per step: 98,304 hexes 35.9, 37.4; 145,800: 44.1, 45.3; 210,000: 72.5, 66.2;
 // 393,216: 131.8, 116.3; 3.84 M: 1,142, 991 (all damaged: 1,633, 1,167).
-constexpr int64_t kPointsFrom = 5 * 4 * 128 * 152 / 2;
+constexpr int64_t kPointsFrom = 5 * 4 * 128 * kSms / 2;
 
 template <typename T>
 void launch_hex(const Dev<T> &D, const Mat<T> &M, cudaStream_t s) {
