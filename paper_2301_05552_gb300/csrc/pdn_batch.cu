@@ -35,8 +35,9 @@ using namespace detail;
 enum TileKind : int32_t { TK_CONTACT = 0, TK_HEX = 1, TK_COH = 2, TK_GATHER = 3, TK_TAIL = 4 };
 
 // The hexes [first, end) of a plate, out of line: the element code then has the
-// launch's whole register budget to itself (inlined into the tile loop it
-// spilled 650 bytes a thread at 128 registers).
+// launch's 128 registers but for the ones the tile loop keeps (84 bytes a thread
+// are spilled in it, and 448 in the dataflow kernel's loop around the calls;
+// inlined it was 650 in the innermost code).
 template <typename T, bool BOX>
 __device__ __noinline__ void batch_hex(const Dev<T> &D, const Mat<T> &M, int64_t first, int64_t end, int mode) {
   hex_item<T, BOX>(D, M, first, end, mode);
